@@ -86,8 +86,8 @@ typedef struct {
                           eight waves of the GPU; either kernel 32 where that fills four,
                           else a balanced split whose grid fills whole waves; a batch: 64
                           staged, 32 generic; D2Q9: 1) */
-  int32_t variant;     /* step kernel: 0 = automatic (staged where it can run), 1 = generic
-                          (any size, any stencil), 2 = cp.async-staged (D3Q19, E4, nx >= 32
+  int32_t variant;     /* step kernel: 0 = automatic (two passes or staged where they can run and are
+                          faster), 1 = generic (any size, any stencil), 2 = cp.async-staged (D3Q19, E4, nx >= 32
                           a multiple of the sites per 16-byte chunk: 1 F64, 2 F32, 4 F16 and
                           BF16; tile_y 4, 8 or 16, F64 tile_y 4 only); both kernels compute
                           the same numbers */
@@ -117,10 +117,12 @@ sc_status sc_create(const sc_params *params, const double *nA0, const double *nB
 
 /* Advance nsteps >= 0 time steps of Eq. lbm (BGK of Eq. omega_i, Guo forcing,
  * equilibrium of Eq. feq, common velocity of Eq. u, force of Eq. sc_force,
- * streaming).  One fused kernel launch per step; asynchronous.  Runs of 32 steps
- * are replayed from a CUDA graph of 32 launches that the context captures once,
- * on a private stream, the first time such a run comes up (the replay goes to the
- * context's stream; if the capture is not possible the steps are plain launches). */
+ * streaming).  One fused kernel launch per step, or two (a moments pass and a
+ * collision pass, the library's choice for small, odd, E6 and FP64 lattices with
+ * tau = 1); asynchronous.  Runs of 32 steps are replayed from a CUDA graph that
+ * the context captures once, on a private stream, the first time such a run comes
+ * up (the replay goes to the context's stream; if the capture is not possible the
+ * steps are plain launches). */
 sc_status sc_step(sc_ctx *ctx, int64_t nsteps);
 
 /* Densities n_A, n_B (device FP64 [N] each) and, if u != NULL, the common
@@ -309,10 +311,14 @@ sc_status sc_run_host_sigma(const sc_params *params, const double *nA0, const do
  * capture).  The kernel is the staged one when every member can take it
  * (variant 0 or 2, D3Q19, E4, nx >= 32 a multiple of the chunk sites; members
  * then share stages and blocks_per_sm), else the generic one; a member with
- * variant 2 in a batch that cannot be staged is an error (SC_EINVAL).
+ * variant 2 in a batch that cannot be staged is an error (SC_EINVAL).  Where every
+ * member leaves variant, tiles and pipeline to the library, is D3Q19 with tau = 1
+ * and has sides >= 4, the batch steps in two passes (a moments and a collision
+ * launch per step, replayed from a CUDA graph) unless a persistent launch is asked
+ * for (sc_batch_set_persistent).
  * By default (where the device has cooperative launch; see
- * sc_batch_set_persistent) a staged batch runs 32 time steps of every member in
- * ONE persistent cooperative launch: in each step its blocks draw the work
+ * sc_batch_set_persistent) a staged batch that does not step in two passes runs 32
+ * time steps of every member in ONE persistent cooperative launch: in each step its blocks draw the work
  * items from a ticket counter, then meet at a grid-wide barrier before the
  * next; a barrier wait that runs out (2^20 polls, a few seconds) sets bit 1 of
  * every member's status word, reported by sc_sync as SC_ETIMEOUT.  Otherwise,
@@ -341,7 +347,7 @@ sc_ctx *sc_batch_member(sc_batch *batch, int32_t k);
  * per step it runs). */
 int64_t sc_batch_launches(const sc_batch *batch);
 /* Step kernel of the batch: 1 generic, 2 staged (one launch per step), 3 staged
- * and persistent (0 for NULL). */
+ * and persistent, 4 two passes (0 for NULL). */
 int32_t sc_batch_variant(const sc_batch *batch);
 /* Stop stepping member k (section 4 runs each droplet until it has converged,
  * so members of a sweep finish at different times).  The member keeps its state
@@ -355,12 +361,13 @@ int32_t sc_batch_active(const sc_batch *batch);
 void sc_batch_destroy(sc_batch *batch);
 
 /* The step kernel this context launches: out[0..8) = variant (1 generic, 2
- * staged), tile_y, tile_z, stages, blocks_per_sm, blocks per launch, balanced
- * split K (0: plain grid of tile_z chunks), columns with K + 1 chunks.  n: room
- * in out (>= 8).  Host only, no synchronisation. */
+ * staged, 3 two passes), tile_y, tile_z, stages, blocks_per_sm, blocks per launch
+ * (of each pass), balanced split K (0: plain grid of tile_z chunks), columns with
+ * K + 1 chunks; with two passes all but the blocks are 0.  n: room in out (>= 8).
+ * Host only, no synchronisation. */
 sc_status sc_step_config(const sc_ctx *ctx, int32_t *out, int32_t n);
 
-/* Number of step-kernel launches issued by this context so far. */
+/* Number of time steps issued by this context so far (a step in two passes counts once). */
 int64_t sc_kernel_launches(const sc_ctx *ctx);
 
 /* Mean initial densities nbar_J used as the storage reference (host out [2]). */

@@ -482,7 +482,7 @@ class Batch:
     @property
     def staged(self) -> bool:
         """True when the batch steps with the staged kernel."""
-        return sc_batch_variant(self.handle) >= 2
+        return sc_batch_variant(self.handle) in (2, 3)
 
     @property
     def persistent(self) -> bool:

@@ -12,6 +12,7 @@
 #include "sc_aux.cuh"
 #include "sc_dispatch.h"
 #include "sc_host.h"
+#include "sc_step_split.cuh"
 
 using namespace scgb;
 
@@ -109,6 +110,25 @@ int default_tile_z(const sc_params *p) {
   return want < p->nz ? want : p->nz;
 }
 
+// The two-pass step can serve these parameters.
+bool split_eligible(const sc_params *p) {
+  return p->lattice == SC_D3Q19 && tau_one(p) && p->nx >= 4 && p->ny >= 4 && p->nz >= 4;
+}
+// ... and does: the step kernel is left to the library (no variant, tile or pipeline asked for), and either
+// the lattice cannot take the staged kernel, or it is FP64 (no density is summed twice), or the moments stay
+// in L2 between the passes.  Staged -> two passes, us a step: FP32 64^3 21.3 -> 11.9, 128^3 120.0 -> 117.6,
+// 160^3 227 -> 227, 256^3 884 -> 887; FP16 96^3 44.3 -> 37.8, 128^3 90.0 -> 91.8 (with a self coupling, whose
+// psi the one-pass kernel evaluates again in every halo, 107.5 -> 96.8, 160^3 185.4 -> 185.9).
+bool split_asked(const sc_params *p) {
+  return split_eligible(p) && !p->variant && !p->tile_y && !p->tile_z && !p->stages && !p->blocks_per_sm;
+}
+bool split_default(const sc_params *p) {
+  if (!split_asked(p)) return false;
+  if (!use_staged(p) || p->storage == SC_STORE_F64) return true;
+  const int64_t sites = (int64_t)p->nx * p->ny * p->nz;
+  return sites <= (is_16bit(p->storage) && !has_self(p) ? int64_t(3) << 19 : int64_t(3) << 20);
+}
+
 sc_status validate(const sc_params *p) {
   sc_status st = validate_model(p);
   if (st != SC_OK) return st;
@@ -159,7 +179,12 @@ Layout layout_of(const sc_params *p) {
   L.off_ref[1] = off;
   off = align_up(off + L.ref_bytes);
   L.off_fields = off;
-  off = align_up(off + (size_t)4 * N * sizeof(double));
+  // the FP64 fields and the moments of the two-pass step share this space: each is computed anew from the
+  // populations before it is read
+  size_t shared = (size_t)4 * N * sizeof(double);
+  if (split_eligible(p))
+    shared = std::max(shared, (size_t)N * (p->storage == SC_STORE_F64 ? 16 : 8) * (has_self(p) ? 5 : 4));
+  off = align_up(off + shared);
   L.off_partial = off;
   off = align_up(off + kPartialBytes);
   L.off_status = off;
@@ -228,6 +253,7 @@ struct sc_ctx {
   int tile_y, tile_z;
   int staged, stages, blocks_per_sm;
   int zbal_k, zbal_rem, zbal_cols, zbal_cols_x;  // balanced z split of the staged kernel (zbal_k > 0)
+  int split;  // the two-pass step (else the one-pass kernels above)
   double nbar[2], psibar[2];
   double scale[2][19], inv_scale[2][19];
   int64_t launches;
@@ -256,6 +282,10 @@ struct sc_batch {
   int active;         // members still stepped
   const void *kernel;
   size_t smem;
+  // the two-pass form: SplitArgs<CT>[n] and (lattice, first site) per block
+  int split, nsplit, stencil, storage;
+  void *sargs_dev;
+  int2 *sitems_dev;
   // the persistent form of the staged batch (one cooperative launch runs kGraphSteps steps of every
   // member; nullptr when the batch is not staged or the device has no cooperative launch)
   const void *pkernel;
@@ -453,6 +483,40 @@ sc_status plan_z_split(sc_ctx *c) {
   return SC_OK;
 }
 
+FastDiv fast_div(unsigned d) {
+  FastDiv f;
+  f.div = d;
+  f.mul = f.shift = 0;
+  if (d > 1) {
+    unsigned l = 1;
+    while ((1ull << l) < d) l++;
+    f.shift = l - 1;
+    f.mul = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
+  }
+  return f;
+}
+
+template <class CT>
+SplitArgs<CT> split_args(sc_ctx *c) {
+  SplitArgs<CT> m;
+  memset(&m, 0, sizeof(m));
+  m.a = step_args<CT>(c);
+  m.mom = reinterpret_cast<P2<CT> *>(fields_of(c));
+  m.dx = fast_div((unsigned)c->p.nx);
+  m.dy = fast_div((unsigned)c->p.ny);
+  return m;
+}
+
+cudaError_t launch_split_step(sc_ctx *c) {
+  const int sten = c->p.stencil == SC_FORCE_E6 ? kE6 : kE4;
+  switch (c->p.storage) {
+    case SC_STORE_F32: return launch_split_f32(sten, split_args<float>(c), c->stream);
+    case SC_STORE_F16: return launch_split_f16(sten, split_args<float>(c), c->stream);
+    case SC_STORE_BF16: return launch_split_bf16(sten, split_args<float>(c), c->stream);
+    default: return launch_split_f64(sten, split_args<double>(c), c->stream);
+  }
+}
+
 sc_status launch_one_step(sc_ctx *c) {
   StepLaunch l;
   l.lattice = c->p.lattice == SC_D3Q19 ? kD3Q19 : kD2Q9;
@@ -464,11 +528,15 @@ sc_status launch_one_step(sc_ctx *c) {
   l.grid = dim3((c->p.nx + 31) / 32, (c->p.ny + c->tile_y - 1) / c->tile_y, (c->p.nz + c->tile_z - 1) / c->tile_z);
   l.stream = c->stream;
   cudaError_t e;
-  switch (c->p.storage) {
-    case SC_STORE_F32: e = launch_step_f32(l, step_args<float>(c)); break;
-    case SC_STORE_F16: e = launch_step_f16(l, step_args<float>(c)); break;
-    case SC_STORE_BF16: e = launch_step_bf16(l, step_args<float>(c)); break;
-    default: e = launch_step_f64(l, step_args<double>(c)); break;
+  if (c->split) {
+    e = launch_split_step(c);
+  } else {
+    switch (c->p.storage) {
+      case SC_STORE_F32: e = launch_step_f32(l, step_args<float>(c)); break;
+      case SC_STORE_F16: e = launch_step_f16(l, step_args<float>(c)); break;
+      case SC_STORE_BF16: e = launch_step_bf16(l, step_args<float>(c)); break;
+      default: e = launch_step_f64(l, step_args<double>(c)); break;
+    }
   }
   if (e != cudaSuccess) return fail(SC_ECUDA, "step kernel launch: %s", cudaGetErrorString(e));
   c->cur = 1 - c->cur;
@@ -562,6 +630,7 @@ sc_status sc_create(const sc_params *params, const double *nA0, const double *nB
   c->stages = effective_stages(params, c->tile_y);
   c->blocks_per_sm = effective_blocks_per_sm(params, c->tile_y);
   c->fields_at = -1;
+  c->split = split_default(params) ? 1 : 0;
   if (params->tile_z == 0 && params->lattice == SC_D3Q19) {
     st = plan_z_split(c);
     if (st != SC_OK) {
@@ -1034,6 +1103,24 @@ sc_params member_params(int32_t n, const sc_params *params, int k, bool staged) 
   return q;
 }
 
+// A batch steps in two passes when every member can and leaves the step kernel to the library, whatever the
+// sizes: the one-pass work list fills whole waves of blocks badly.  Us a step, persistent staged (generic for
+// the paper's odd sides) -> two passes: 16 droplets, 22.1 M sites FP32 1296 -> 1231, FP16 1088 -> 1071, BF16
+// 1054 -> 1040; 4 droplets, 0.29 M sites FP32 131 -> 14.6; 14 paper droplets, 1.5 M sites FP32 160 -> 101.
+bool batch_split(int32_t n, const sc_params *params) {
+  for (int k = 0; k < n; ++k)
+    if (!split_asked(&params[k])) return false;
+  return true;
+}
+// Its tables: SplitArgs of the members, then the items.
+size_t split_table_bytes(int32_t n, const sc_params *params, int64_t *items_out) {
+  int64_t items = 0;
+  for (int k = 0; k < n; ++k)
+    items += ((int64_t)params[k].nx * params[k].ny * params[k].nz + kSplitBatchSites - 1) / kSplitBatchSites;
+  if (items_out) *items_out = items;
+  return align_up(sizeof(SplitArgs<double>) * (size_t)n) + align_up(sizeof(int2) * (size_t)items);
+}
+
 size_t batch_table_bytes(int32_t n, const sc_params *params, int *nitems_out) {
   const bool staged = batch_staged(n, params);
   int nitems = 0;
@@ -1043,7 +1130,8 @@ size_t batch_table_bytes(int32_t n, const sc_params *params, int *nitems_out) {
     nitems += ((q.nx + 31) / 32) * ((q.ny + ty - 1) / ty) * ((q.nz + tz - 1) / tz);
   }
   if (nitems_out) *nitems_out = nitems;
-  return align_up(sizeof(StepArgs<double>) * (size_t)n) + align_up(sizeof(int4) * (size_t)nitems) + kAlign;
+  return align_up(sizeof(StepArgs<double>) * (size_t)n) + align_up(sizeof(int4) * (size_t)nitems) + kAlign +
+         (batch_split(n, params) ? split_table_bytes(n, params, nullptr) : 0);
 }
 
 sc_status batch_validate(int32_t n, const sc_params *params) {
@@ -1082,7 +1170,24 @@ sc_status batch_upload_items(sc_batch *b) {
     total += ((c->p.nx + 31) / 32) * ((c->p.ny + c->tile_y - 1) / c->tile_y) * ((c->p.nz + c->tile_z - 1) / c->tile_z);
   }
   b->nitems = total;
+  b->nsplit = 0;
   if (total == 0) return SC_OK;
+  if (b->sitems_dev) {
+    int64_t count = 0;
+    for (int k = 0; k < b->n; ++k)
+      if (!b->retired[k]) count += (b->ctx[k]->N + kSplitBatchSites - 1) / kSplitBatchSites;
+    int2 *si = new (std::nothrow) int2[count];
+    if (!si) return fail(SC_ENOMEM, "host allocation failed");
+    int64_t q = 0;
+    for (int k = 0; k < b->n; ++k)
+      if (!b->retired[k])
+        for (int64_t s = 0; s < b->ctx[k]->N; s += kSplitBatchSites) si[q++] = make_int2(k, (int)s);
+    cudaError_t e = cudaMemcpyAsync(b->sitems_dev, si, sizeof(int2) * count, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    delete[] si;
+    if (e != cudaSuccess) return fail(SC_ECUDA, "uploading the batch work list: %s", cudaGetErrorString(e));
+    b->nsplit = (int)count;
+  }
   int4 *items = new (std::nothrow) int4[total];
   if (!items) return fail(SC_ENOMEM, "host allocation failed");
   int m = 0;
@@ -1162,6 +1267,37 @@ bool batch_build_persistent(sc_batch *b) {
   return true;
 }
 
+// One time step of a two-pass batch on stream st.
+cudaError_t batch_split_step(const sc_batch *b, int swap, cudaStream_t st) {
+  switch (b->storage) {
+    case SC_STORE_F32:
+      return launch_split_batch_f32(b->stencil, static_cast<SplitArgs<float> *>(b->sargs_dev), b->sitems_dev, b->nsplit, swap, st);
+    case SC_STORE_F16:
+      return launch_split_batch_f16(b->stencil, static_cast<SplitArgs<float> *>(b->sargs_dev), b->sitems_dev, b->nsplit, swap, st);
+    case SC_STORE_BF16:
+      return launch_split_batch_bf16(b->stencil, static_cast<SplitArgs<float> *>(b->sargs_dev), b->sitems_dev, b->nsplit, swap, st);
+    default:
+      return launch_split_batch_f64(b->stencil, static_cast<SplitArgs<double> *>(b->sargs_dev), b->sitems_dev, b->nsplit, swap, st);
+  }
+}
+
+// kGraphSteps steps of a two-pass batch, captured on a private stream (the launches' programmatic
+// dependences are kept as edges of the graph).
+cudaError_t batch_capture_split(sc_batch *b) {
+  cudaStream_t st = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed);
+  if (e == cudaSuccess) {
+    for (int t = 0; t < kGraphSteps && e == cudaSuccess; ++t) e = batch_split_step(b, t & 1, st);
+    const cudaError_t ended = cudaStreamEndCapture(st, &b->graph);
+    if (e == cudaSuccess) e = ended;
+  }
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
+  cudaStreamDestroy(st);
+  return e;
+}
+
 // A graph of kGraphSteps steps over the current work list, swap = 0, 1, 0, 1, ...: the persistent
 // form where the batch has one, else kGraphSteps chained launches (none when no member is left).
 sc_status batch_build_graph(sc_batch *b) {
@@ -1171,6 +1307,11 @@ sc_status batch_build_graph(sc_batch *b) {
   b->graph = nullptr;
   b->pgrid = 0;
   if (b->nitems == 0) return SC_OK;
+  if (b->split) {
+    const cudaError_t e = batch_capture_split(b);
+    if (e != cudaSuccess) return fail(SC_ECUDA, "building the batch graph: %s", cudaGetErrorString(e));
+    return SC_OK;
+  }
   if (b->pkernel && !b->persist_off && batch_build_persistent(b)) return SC_OK;
   cudaError_t e = cudaGraphCreate(&b->graph, 0);
   cudaGraphNode_t prev = nullptr;
@@ -1248,7 +1389,15 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
   b->items_dev = reinterpret_cast<int4 *>(ws + off);
   off += align_up(sizeof(int4) * (size_t)nitems);
   b->counter = reinterpret_cast<unsigned *>(ws + off);
+  off += kAlign;
   const int storage = params[0].storage;
+  b->storage = storage;
+  b->stencil = params[0].stencil == SC_FORCE_E6 ? kE6 : kE4;
+  b->split = batch_split(n, params) ? 1 : 0;
+  if (b->split) {
+    b->sargs_dev = ws + off;
+    b->sitems_dev = reinterpret_cast<int2 *>(ws + off + align_up(sizeof(SplitArgs<double>) * (size_t)n));
+  }
   const size_t arg_size = storage == SC_STORE_F64 ? sizeof(StepArgs<double>) : sizeof(StepArgs<float>);
   std::string host_args(arg_size * n, '\0');
   for (int k = 0; k < n; ++k) {
@@ -1261,7 +1410,22 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
       memcpy(&host_args[arg_size * k], &a, arg_size);
     }
   }
+  std::string host_split;
+  if (b->split) {
+    const size_t size = storage == SC_STORE_F64 ? sizeof(SplitArgs<double>) : sizeof(SplitArgs<float>);
+    for (int k = 0; k < n; ++k) {
+      if (storage == SC_STORE_F64) {
+        const SplitArgs<double> a = split_args<double>(b->ctx[k]);
+        host_split.append(reinterpret_cast<const char *>(&a), size);
+      } else {
+        const SplitArgs<float> a = split_args<float>(b->ctx[k]);
+        host_split.append(reinterpret_cast<const char *>(&a), size);
+      }
+    }
+  }
   cudaError_t e = cudaMemcpyAsync(b->args_dev, host_args.data(), arg_size * n, cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess && b->split)
+    e = cudaMemcpyAsync(b->sargs_dev, host_split.data(), host_split.size(), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {
     sc_batch_destroy(b);
@@ -1335,6 +1499,12 @@ sc_status sc_batch_step(sc_batch *b, int64_t nsteps) {
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
   if (b->nitems == 0) return SC_OK;  // every member retired
   auto single = [&]() -> cudaError_t {
+    if (b->split) {
+      const cudaError_t e = batch_split_step(b, (int)(b->steps & 1), b->stream);
+      b->steps++;
+      b->launches++;
+      return e;
+    }
     void *argp = b->args_dev;
     void *itemp = b->items_dev;
     int swap = (int)(b->steps & 1);
@@ -1384,8 +1554,10 @@ sc_status sc_batch_set_persistent(sc_batch *b, int32_t on) {
   if (!b) return fail(SC_EINVAL, "batch is NULL");
   if (on != 0 && on != 1) return fail(SC_EINVAL, "on must be 0 or 1");
   if (on && !b->pkernel) return fail(SC_EUNSUPPORTED, "the batch has no persistent form (generic kernel or no cooperative launch)");
+  if (b->split && !on) return SC_OK;  // no persistent launch in use
   SC_CUDA(cudaStreamSynchronize(b->stream));
   b->persist_off = !on;
+  b->split = 0;
   sc_status st = batch_build_graph(b);
   if (st == SC_OK && on && b->nitems > 0 && b->pgrid == 0)
     return fail(SC_EUNSUPPORTED, "the persistent launch could not be built on this device");
@@ -1401,7 +1573,11 @@ sc_ctx *sc_batch_member(sc_batch *b, int32_t k) {
 }
 
 int64_t sc_batch_launches(const sc_batch *b) { return b ? b->launches : 0; }
-int32_t sc_batch_variant(const sc_batch *b) { return b ? (b->staged ? (b->pgrid > 0 ? 3 : 2) : 1) : 0; }
+int32_t sc_batch_variant(const sc_batch *b) {
+  if (!b) return 0;
+  if (b->split) return 4;
+  return b->staged ? (b->pgrid > 0 ? 3 : 2) : 1;
+}
 
 void sc_batch_destroy(sc_batch *b) {
   if (!b) return;
@@ -1420,6 +1596,11 @@ sc_status sc_step_config(const sc_ctx *c, int32_t *out, int32_t n) {
   const int64_t grid = c->zbal_k > 0 ? (int64_t)c->zbal_k * c->zbal_cols + c->zbal_rem
                                      : (int64_t)((c->p.nx + 31) / 32) * ((c->p.ny + c->tile_y - 1) / c->tile_y) *
                                            ((c->p.nz + c->tile_z - 1) / c->tile_z);
+  if (c->split) {
+    const int32_t v[8] = {3, 0, 0, 0, 0, (int32_t)((c->N + kSplitThreads - 1) / kSplitThreads), 0, 0};
+    for (int k = 0; k < 8; ++k) out[k] = v[k];
+    return SC_OK;
+  }
   const int32_t v[8] = {c->staged ? 2 : 1, c->tile_y, c->tile_z, c->staged ? c->stages : 0,
                         c->staged ? c->blocks_per_sm : 0, (int32_t)grid, c->zbal_k, c->zbal_rem};
   for (int k = 0; k < 8; ++k) out[k] = v[k];

@@ -76,4 +76,21 @@ const void *persistent_staged_kernel_f64(int tile_y, int stages, int blocks_per_
 // completes): zeroes *counter, then the wait runs out after max_polls polls and sets bit 1 of *err.
 cudaError_t launch_barrier_probe(unsigned *counter, unsigned *err, unsigned max_polls, cudaStream_t st);
 
+// One time step in two passes (sc_step_split.cuh): of one lattice, or of the lattices of a batch over its
+// items (lattice, first site).
+template <class CT>
+struct SplitArgs;
+cudaError_t launch_split_f32(int stencil, const SplitArgs<float> &m, cudaStream_t st);
+cudaError_t launch_split_batch_f32(int stencil, const SplitArgs<float> *args, const int2 *items, int nitems, int swap,
+                                   cudaStream_t st);
+cudaError_t launch_split_f16(int stencil, const SplitArgs<float> &m, cudaStream_t st);
+cudaError_t launch_split_batch_f16(int stencil, const SplitArgs<float> *args, const int2 *items, int nitems, int swap,
+                                   cudaStream_t st);
+cudaError_t launch_split_bf16(int stencil, const SplitArgs<float> &m, cudaStream_t st);
+cudaError_t launch_split_batch_bf16(int stencil, const SplitArgs<float> *args, const int2 *items, int nitems, int swap,
+                                   cudaStream_t st);
+cudaError_t launch_split_f64(int stencil, const SplitArgs<double> &m, cudaStream_t st);
+cudaError_t launch_split_batch_f64(int stencil, const SplitArgs<double> *args, const int2 *items, int nitems, int swap,
+                                   cudaStream_t st);
+
 }  // namespace scgb

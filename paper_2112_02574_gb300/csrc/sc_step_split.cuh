@@ -1,0 +1,214 @@
+// The time step in two passes (D3Q19, E4 or E6, tau_A = tau_B = 1, every side >= 4, any storage).
+//
+//  * The moments pass pulls the populations of a site once and keeps what collisions need of them:
+//    the density deviation pair, the three momentum-sum pairs (carry_size) and, with a self coupling,
+//    the psi deviation pair.
+//  * The collision pass reads those of the site, the density (and psi) of its stencil neighbours, and
+//    writes the post-collision populations.
+//
+// The arithmetic is that of sc_step_kernel, operation by operation, so the stored bits are the same.
+// Against the one-pass kernels no density is summed twice (they re-sum a halo of one or two sites around
+// every tile and chunk, and evaluate psi there), a thread takes one site of the linear order whatever the
+// sides are (no lane idles in a partial x tile), and no block waits at a barrier; in return 32 bytes a site
+// (40 with a self coupling; twice that in FP64) are written and read again between the passes, through L2
+// while that buffer fits there.
+// Measured, one step, one-pass -> two passes (FP32 unless noted): E6 64 x 64 x 256 80.3 -> 68.2 us,
+// E6 160^3 302 -> 259 us (FP16 363 -> 209 us), 65^3 29.5 -> 15.1 us (paper couplings), 201^3 567 -> 497 us,
+// 64^3 21.4 -> 11.9 us, FP64 64^3 284 -> 191 us.  Bound: HBM at large sizes (256^3: 368 bytes a site at
+// 6.9 TB/s), FP64 arithmetic in FP64, latency below about 40^3.
+#pragma once
+
+#include "sc_step_kernel.cuh"
+
+namespace scgb {
+
+// Exact quotient of 0 <= n < 2^31 by a fixed divisor: mul = ceil(2^(32 + shift) / div), shift =
+// ceil(log2 div) - 1, so that the rounding of mul adds less than 1 / div to n / div.
+struct FastDiv {
+  unsigned mul, shift, div;
+  __host__ __device__ __forceinline__ unsigned quot(unsigned n) const {
+    return div == 1 ? n : (unsigned)(((unsigned long long)n * mul) >> 32) >> shift;
+  }
+};
+
+// One lattice as the two passes step it.
+template <class CT>
+struct SplitArgs {
+  StepArgs<CT> a;
+  P2<CT> *mom;  // [4 or 5][N]: density deviation, momentum sums x, y, z, with a self coupling psi deviation
+  FastDiv dx, dy;
+};
+
+// Launches follow one another as programmatic dependents: a pass starts while the one before drains, and
+// waits here before its first access to what that one wrote.  The launch of the next pass is allowed only
+// after the wait, so that at most two passes are on the device and no pass starts (and caches lines in L1)
+// before the last but one is complete; no load goes through the read-only path, whose data must not change
+// while a kernel runs.
+__device__ __forceinline__ void pass_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class CT>
+__device__ __forceinline__ void split_coords(const SplitArgs<CT> &m, int s, int &x, int &y, int &z) {
+  const unsigned q = m.dx.quot((unsigned)s);
+  x = s - (int)q * m.a.nx;
+  z = (int)m.dy.quot(q);
+  y = (int)q - z * m.a.ny;
+}
+
+// Moments pass at site s.
+template <class ST, class CT>
+__device__ __forceinline__ void split_moments(const SplitArgs<CT> &m, const ST *src, const float2 *nsrc, int s) {
+  using L = Lattice<kD3Q19>;
+  const StepArgs<CT> &a = m.a;
+  int x, y, z;
+  split_coords<CT>(m, s, x, y, z);
+  // site offset of the source for a velocity component of -1, 0, +1
+  const int W = a.nx * a.ny;
+  const int X[3] = {x == a.nx - 1 ? 1 - a.nx : 1, 0, x == 0 ? a.nx - 1 : -1};
+  const int Y[3] = {y == a.ny - 1 ? a.nx * (1 - a.ny) : a.nx, 0, y == 0 ? a.nx * (a.ny - 1) : -a.nx};
+  const int Z[3] = {z == a.nz - 1 ? W * (1 - a.nz) : W, 0, z == 0 ? W * (a.nz - 1) : -W};
+  P2<CT> g[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const int site = s + X[L::c(i, 0) + 1] + Y[L::c(i, 1) + 1] + Z[L::c(i, 2) + 1];
+    g[i] = Codec2<ST, CT>::template load<true>(src + ((int64_t)i * a.N + site) * 2, a.inv_scale);
+    if constexpr (local_ref<ST>()) {
+      const float2 ns = nsrc[site];
+      g[i] = pfma(wpair<kD3Q19, ST, CT>(i, a.scale), pset(CT(ns.x), CT(ns.y)), g[i]);
+    }
+  }
+  P2<CT> sum = pbc(CT(0));
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) sum = padd(sum, g[i]);
+  const P2<CT> dn = unscale<ST, CT>(sum, a.inv_scale);
+  P2<CT> j[3];
+  momentum_sums<kD3Q19, CT>(g, j);
+  m.mom[s] = dn;
+  m.mom[a.N + s] = j[0];
+  m.mom[2 * a.N + s] = j[1];
+  m.mom[3 * a.N + s] = j[2];
+  if (a.self_on) m.mom[4 * a.N + s] = psi_deviation<CT>(dn, a.nbar, a.psibar, a.psi_exp, a.gself);
+}
+
+// Collision pass at site s: Eq. sc_force from the stored densities in force_pair's order, then the shared collision.
+template <int STEN, class ST, class CT>
+__device__ __forceinline__ void split_collide(const SplitArgs<CT> &m, ST *dst, float2 *ndst, int s) {
+  using L = Lattice<kD3Q19>;
+  using SN = Stencil<kD3Q19, STEN>;
+  constexpr int H = SN::HALO;
+  const StepArgs<CT> &a = m.a;
+  int x, y, z;
+  split_coords<CT>(m, s, x, y, z);
+  const P2<CT> *dnp = m.mom, *psp = m.mom + 4 * a.N;
+  const P2<CT> j[3] = {m.mom[a.N + s], m.mom[2 * a.N + s], m.mom[3 * a.N + s]};
+  const P2<CT> dn = dnp[s];
+  const P2<CT> n = padd(a.nbar, dn);
+  int X[2 * H + 1], Y[2 * H + 1], Z[2 * H + 1];
+  const int W = a.nx * a.ny;
+#pragma unroll
+  for (int d = -H; d <= H; ++d) {
+    X[d + H] = wrapi(x + d, a.nx) - x;
+    Y[d + H] = (wrapi(y + d, a.ny) - y) * a.nx;
+    Z[d + H] = (wrapi(z + d, a.nz) - z) * W;
+  }
+  P2<CT> S[3] = {pbc(CT(0)), pbc(CT(0)), pbc(CT(0))}, T[3] = {pbc(CT(0)), pbc(CT(0)), pbc(CT(0))};
+#pragma unroll
+  for (int k = 0; k < SN::NH; ++k) {
+    const int vx = SN::v(k, 0), vy = SN::v(k, 1), vz = SN::v(k, 2);
+    const int ip = s + X[H + vx] + Y[H + vy] + Z[H + vz], im = s + X[H - vx] + Y[H - vy] + Z[H - vz];
+    const P2<CT> d = psub(dnp[ip], dnp[im]);
+    if (vx) S[0] = pfma(pbc(CT(SN::W(k) * vx)), d, S[0]);
+    if (vy) S[1] = pfma(pbc(CT(SN::W(k) * vy)), d, S[1]);
+    if (vz) S[2] = pfma(pbc(CT(SN::W(k) * vz)), d, S[2]);
+    if (a.self_on) {
+      const P2<CT> e = psub(psp[ip], psp[im]);
+      if (vx) T[0] = pfma(pbc(CT(SN::W(k) * vx)), e, T[0]);
+      if (vy) T[1] = pfma(pbc(CT(SN::W(k) * vy)), e, T[1]);
+      if (vz) T[2] = pfma(pbc(CT(SN::W(k) * vz)), e, T[2]);
+    }
+  }
+  const P2<CT> psi = a.self_on ? padd(a.psibar, psp[s]) : pbc(CT(0));
+  const P2<CT> cn = pmul(pbc(a.gcross), n), cp = pmul(a.gself, psi);
+  P2<CT> F[3], h[3], out[L::Q];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) F[q] = pfma(cp, T[q], pmul(cn, pswap(S[q])));
+  CT u[3];
+  half_momentum<ST, CT>(j, F, a.inv_scale, h);
+  common_velocity<CT>(h, n, u);
+  collide_pair<kD3Q19, ST, CT, true>(a, nullptr, n, dn, u, F, out);
+  check_density<CT>(a, n);
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) Codec2<ST, CT>::store(dst + ((int64_t)i * a.N + s) * 2, out[i], a.scale);
+  if constexpr (local_ref<ST>()) ndst[s] = make_float2(float(dn.x), float(dn.y));
+}
+
+// Threads per block and the blocks per SM the register allocation must allow (64 registers a thread, 80 for
+// the 33 neighbours of E6 in a batch, which would spill; 128 in FP64).  128 threads against 256: 1-2 %
+// faster from 64^3 up, equal below.
+constexpr int kSplitThreads = 128;
+template <class CT>
+constexpr int split_blocks(bool spills = false) { return sizeof(CT) == 8 ? 4 : (spills ? 6 : 8); }
+
+template <class ST, class CT>
+__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>())
+    sc_split_moments(const __grid_constant__ SplitArgs<CT> m) {
+  const int s = blockIdx.x * kSplitThreads + threadIdx.x;
+  pass_begin();
+  if (s < m.a.N) split_moments<ST, CT>(m, static_cast<const ST *>(m.a.src), m.a.nsrc, s);
+}
+
+template <int STEN, class ST, class CT>
+__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>())
+    sc_split_collide(const __grid_constant__ SplitArgs<CT> m) {
+  const int s = blockIdx.x * kSplitThreads + threadIdx.x;
+  pass_begin();
+  if (s < m.a.N) split_collide<STEN, ST, CT>(m, static_cast<ST *>(m.a.dst), m.a.ndst, s);
+}
+
+// Batched forms: block b takes kSplitBatchSites sites from site items[b].y of lattice items[b].x (the arguments
+// args[lattice] in shared memory), source and destination swapped when swap != 0.  Two sites a thread: the
+// fetch of the item and the arguments is paid once for both.
+constexpr int kSplitBatchSites = 2 * kSplitThreads;
+
+template <class CT>
+__device__ __forceinline__ void split_fetch(SplitArgs<CT> &m, const SplitArgs<CT> *args, int lat) {
+  static_assert(sizeof(SplitArgs<CT>) % 4 == 0 && sizeof(SplitArgs<CT>) <= 4 * 2 * kSplitThreads, "copied by words");
+  const int *from = reinterpret_cast<const int *>(args + lat);
+  int *to = reinterpret_cast<int *>(&m);
+  for (int k = threadIdx.x; k < (int)(sizeof(SplitArgs<CT>) / 4); k += kSplitThreads) to[k] = from[k];
+  __syncthreads();
+}
+
+template <class ST, class CT>
+__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>())
+    sc_split_moments_batched(const SplitArgs<CT> *args, const int2 *items, int swap) {
+  __shared__ SplitArgs<CT> m;
+  const int2 it = items[blockIdx.x];
+  split_fetch<CT>(m, args, it.x);
+  pass_begin();
+  const ST *src = static_cast<const ST *>(swap ? m.a.dst : m.a.src);
+  const float2 *nsrc = swap ? m.a.ndst : m.a.nsrc;
+  for (int k = 0; k < kSplitBatchSites; k += kSplitThreads) {
+    const int64_t s = (int64_t)it.y + k + threadIdx.x;
+    if (s < m.a.N) split_moments<ST, CT>(m, src, nsrc, (int)s);
+  }
+}
+
+template <int STEN, class ST, class CT>
+__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>(STEN == kE6))
+    sc_split_collide_batched(const SplitArgs<CT> *args, const int2 *items, int swap) {
+  __shared__ SplitArgs<CT> m;
+  const int2 it = items[blockIdx.x];
+  split_fetch<CT>(m, args, it.x);
+  pass_begin();
+  ST *dst = static_cast<ST *>(swap ? const_cast<void *>(m.a.src) : m.a.dst);
+  float2 *ndst = swap ? const_cast<float2 *>(m.a.nsrc) : m.a.ndst;
+  for (int k = 0; k < kSplitBatchSites; k += kSplitThreads) {
+    const int64_t s = (int64_t)it.y + k + threadIdx.x;
+    if (s < m.a.N) split_collide<STEN, ST, CT>(m, dst, ndst, (int)s);
+  }
+}
+
+}  // namespace scgb
