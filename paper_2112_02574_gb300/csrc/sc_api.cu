@@ -198,6 +198,26 @@ Layout layout_of(const sc_params *p) {
 
 }  // namespace
 
+FastDiv scgb::fast_div(unsigned d) {
+  FastDiv f;
+  f.div = d;
+  f.mul = f.shift = 0;
+  if (d > 1) {
+    unsigned l = 1;
+    while ((1ull << l) < d) l++;
+    f.shift = l - 1;
+    f.mul = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
+  }
+  return f;
+}
+
+SiteDiv scgb::site_div(const sc_params *p) {
+  SiteDiv d;
+  d.dx = fast_div((unsigned)p->nx);
+  d.dy = fast_div((unsigned)p->ny);
+  return d;
+}
+
 // Records the calling thread's sc_last_error() message for entry points defined
 // in other translation units of the library.
 sc_status scgb::set_error(sc_status st, const char *msg) { return fail(st, "%s", msg); }
@@ -316,6 +336,7 @@ PopArgs pop_args(sc_ctx *c, int buf) {
   a.ny = c->p.ny;
   a.nz = c->p.nz;
   a.N = c->N;
+  a.div = site_div(&c->p);
   for (int J = 0; J < 2; ++J) {
     a.nbar[J] = c->nbar[J];
     for (int i = 0; i < 19; ++i) {
@@ -335,6 +356,7 @@ ForceParams force_params(const sc_ctx *c) {
   f.ny = c->p.ny;
   f.nz = c->p.nz;
   f.N = c->N;
+  f.div = site_div(&c->p);
   return f;
 }
 
@@ -366,7 +388,8 @@ int grid_for(int64_t n, int block) {
 sc_status ensure_fields(sc_ctx *c) {
   if (c->fields_at == c->steps) return SC_OK;
   PopArgs a = pop_args(c, c->cur);
-  SC_POP_DISPATCH(c, fields_kernel, grid_for(c->N, 256), 256, 0, a, c->p.psi_self, fields_of(c));
+  SC_POP_DISPATCH(c, fields_kernel, grid_for(c->N, 128), 128, 0, a, c->p.psi_self,
+                  (c->p.G_self[0] != 0.0 ? 1 : 0) | (c->p.G_self[1] != 0.0 ? 2 : 0), fields_of(c));
   SC_CUDA(cudaGetLastError());
   c->fields_at = c->steps;
   return SC_OK;
@@ -483,27 +506,13 @@ sc_status plan_z_split(sc_ctx *c) {
   return SC_OK;
 }
 
-FastDiv fast_div(unsigned d) {
-  FastDiv f;
-  f.div = d;
-  f.mul = f.shift = 0;
-  if (d > 1) {
-    unsigned l = 1;
-    while ((1ull << l) < d) l++;
-    f.shift = l - 1;
-    f.mul = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
-  }
-  return f;
-}
-
 template <class CT>
 SplitArgs<CT> split_args(sc_ctx *c) {
   SplitArgs<CT> m;
   memset(&m, 0, sizeof(m));
   m.a = step_args<CT>(c);
   m.mom = reinterpret_cast<P2<CT> *>(fields_of(c));
-  m.dx = fast_div((unsigned)c->p.nx);
-  m.dy = fast_div((unsigned)c->p.ny);
+  m.div = site_div(&c->p);
   return m;
 }
 
@@ -565,7 +574,7 @@ sc_status init_reductions(sc_ctx *c, const double *nA0, const double *nB0, doubl
   free(mins);
   if (bad) return fail(SC_EINVAL, "initial densities must be finite and > 0");
   sum2_partial_kernel<<<blocks, 256, 0, c->stream>>>(nA0, nB0, c->N, part);
-  totals_finalize_kernel<<<1, 32, 0, c->stream>>>(part, blocks, 2, sc);
+  totals_finalize_kernel<2><<<1, 256, 0, c->stream>>>(part, blocks, sc);
   SC_CUDA(cudaGetLastError());
   SC_CUDA(cudaMemcpyAsync(mean, sc, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   SC_CUDA(cudaStreamSynchronize(c->stream));
@@ -797,7 +806,7 @@ sc_status sc_velocity_change(sc_ctx *c, double *u_prev, double *out) {
   if (lat == SC_D2Q9) SC_DU_ST(kD2Q9, kE4);
 #undef SC_DU_ST
 #undef SC_DU
-  finalize_measure_kernel<<<1, 32, 0, c->stream>>>(part, blocks, 0, 1.0 / double(c->N), out);
+  finalize_sum_kernel<1><<<1, 256, 0, c->stream>>>(part, blocks, 1.0 / double(c->N), out);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }
@@ -810,9 +819,9 @@ sc_status sc_centre_of_mass(sc_ctx *c, int32_t component, double background, dou
   if (st != SC_OK) return st;
   const int blocks = grid_for(c->N, 256) < kMaxPartialBlocks ? grid_for(c->N, 256) : kMaxPartialBlocks;
   double *part = partial_of(c);
-  com_partial_kernel<<<blocks, 256, 0, c->stream>>>(fields_of(c) + (int64_t)component * c->N, c->p.nx, c->p.ny, c->N,
-                                                    background, part);
-  finalize_measure_kernel<<<1, 32, 0, c->stream>>>(part, blocks, 1, 1.0, out);
+  com_partial_kernel<<<blocks, 256, 0, c->stream>>>(fields_of(c) + (int64_t)component * c->N, c->p.nx, c->p.ny, site_div(&c->p),
+                                                    c->N, background, part);
+  finalize_com_kernel<<<1, 256, 0, c->stream>>>(part, blocks, out);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }
@@ -880,7 +889,7 @@ sc_status sc_bulk_pressure_at(sc_ctx *c, const int32_t node[3], double *out) {
   sc_status st = ensure_fields(c);
   if (st != SC_OK) return st;
   const int64_t s = (int64_t)node[0] + (int64_t)c->p.nx * (node[1] + (int64_t)c->p.ny * node[2]);
-  bulk_pressure_kernel<<<1, 32, 0, c->stream>>>(force_params(c), fields_of(c), s, out);
+  bulk_pressure_kernel<<<1, 32, 0, c->stream>>>(force_params(c), fields_of(c), s, -1, out);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }
@@ -892,7 +901,7 @@ sc_status sc_sigma_minimum(const double *rows, int32_t nbins, const double *P_in
   if (dim != 2 && dim != 3) return fail(SC_EINVAL, "dim must be 2 or 3");
   if (!(R_lo > 0.0) || !(R_hi > R_lo) || !(R_step > 0.0) || (R_hi - R_lo) / R_step > 1e7)
     return fail(SC_EINVAL, "need 0 < R_lo < R_hi, R_step > 0 and at most 1e7 grid points");
-  sigma_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(rows, nbins, P_in_out, dim, R_lo, R_hi, R_step, out);
+  sigma_kernel<<<1, kSigmaThreads, 0, static_cast<cudaStream_t>(stream)>>>(rows, nbins, P_in_out, dim, R_lo, R_hi, R_step, out);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }
@@ -926,16 +935,15 @@ sc_status sc_surface_of_tension(sc_ctx *c, int32_t kind, const double centre[3],
   st = sc_pressure_profile(c, kind, ctr, bin_width, nbins, r);
   if (st != SC_OK) return st;
   // P_in at the centre node, P_out at the far corner (section 4)
-  int32_t in_node[3], out_node[3];
+  int64_t in_node[3];
   for (int m = 0; m < 3; ++m) {
     const int k = (int)floor(ctr[m] + 0.5);
     in_node[m] = ((k % nn[m]) + nn[m]) % nn[m];
-    out_node[m] = nn[m] - 1;
   }
   double *pio = analysis_pio(c);
-  st = sc_bulk_pressure_at(c, in_node, pio);
-  if (st == SC_OK) st = sc_bulk_pressure_at(c, out_node, pio + 1);
-  if (st != SC_OK) return st;
+  bulk_pressure_kernel<<<1, 32, 0, c->stream>>>(force_params(c), fields_of(c),
+                                                in_node[0] + nn[0] * (in_node[1] + nn[1] * in_node[2]), c->N - 1, pio);
+  SC_CUDA(cudaGetLastError());
   return sc_sigma_minimum(r, nbins, pio, dim, R_lo, R_hi, R_step, out, c->stream);
 }
 
@@ -980,7 +988,7 @@ sc_status sc_totals(sc_ctx *c, double *out) {
   const int blocks = grid_for(c->N, 256) < kMaxPartialBlocks ? grid_for(c->N, 256) : kMaxPartialBlocks;
   PopArgs a = pop_args(c, c->cur);
   SC_POP_DISPATCH(c, totals_partial_kernel, blocks, 256, 0, a, partial_of(c));
-  totals_finalize_kernel<<<1, 32, 0, c->stream>>>(partial_of(c), blocks, 5, out);
+  totals_finalize_kernel<5><<<1, 256, 0, c->stream>>>(partial_of(c), blocks, out);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }

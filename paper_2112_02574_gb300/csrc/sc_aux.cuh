@@ -41,6 +41,7 @@ struct PopArgs {
   float2 *nref;      // local reference density deviations n_ref - nbar [N] (16-bit storage; nullptr otherwise)
   int nx, ny, nz;
   int64_t N;
+  SiteDiv div;
   double nbar[2];
   double scale[2][19];
   double inv_scale[2][19];
@@ -110,96 +111,193 @@ __global__ void pop_kernel(PopArgs a, int mode, const double *n0A, const double 
   }
 }
 
-// FP64 density fields n_J (and psi_J) from the stored state (pull + sum).
-// fields: [4][N] = n_A, n_B, psi_A, psi_B.
-template <int LAT, class ST>
-__global__ void fields_kernel(PopArgs a, int psi_exp, double *fields) {
+// Exact-to-FP64 sums of FP32 pairs.  GB300 issues one FP64 warp instruction per 16 cycles and SM but four FP32
+// ones per cycle, so sums of values that are stored in FP32 (or fewer bits) are kept as three FP32 terms: each
+// addition is Knuth's TwoSum (an error-free transformation) with the error passed down, so that what is dropped is
+// below 2^-70 of the sum, and only the result is converted.  Against FP64 sums of the 38 populations of a site
+// (38 conversions, 38 additions): density fields of 128^3 FP32 647 -> 88 us, BF16 with one psi 1062 -> 197 us,
+// velocity BF16 1929 -> 683 us (its force stays FP64).
+struct PairSum3 {
+  float2 a = {0.0f, 0.0f}, b = {0.0f, 0.0f}, c = {0.0f, 0.0f};
+  __device__ __forceinline__ static float2 neg_add(float2 x, float2 y) {  // x - y
+    return __ffma2_rn(y, make_float2(-1.0f, -1.0f), x);
+  }
+  __device__ __forceinline__ static float2 two_sum(float2 &s, float2 v) {  // s += v, returns the error
+    const float2 t = __fadd2_rn(s, v), bb = neg_add(t, s);
+    const float2 e = __fadd2_rn(neg_add(s, neg_add(t, bb)), neg_add(v, bb));
+    s = t;
+    return e;
+  }
+  __device__ __forceinline__ void add(float2 v) { c = __fadd2_rn(c, two_sum(b, two_sum(a, v))); }
+  __device__ __forceinline__ void sub(float2 v) { add(make_float2(-v.x, -v.y)); }
+  __device__ __forceinline__ double2 value() const {
+    return make_double2(((double)c.x + (double)b.x) + (double)a.x, ((double)c.y + (double)b.y) + (double)a.y);
+  }
+};
+struct PairSumD {
+  double2 s = {0.0, 0.0};
+  __device__ __forceinline__ void add(double2 v) { s = padd(s, v); }
+  __device__ __forceinline__ void sub(double2 v) { s = psub(s, v); }
+  __device__ __forceinline__ double2 value() const { return s; }
+};
+template <class ST>
+using PairSum = std::conditional_t<std::is_same<ST, double>::value, PairSumD, PairSum3>;
+template <class ST>
+using PairOf = std::conditional_t<std::is_same<ST, double>::value, double, float>;
+
+__device__ __forceinline__ float2 stored_pair(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+__device__ __forceinline__ double2 stored_pair(const double *p) { return *reinterpret_cast<const double2 *>(p); }
+__device__ __forceinline__ float2 stored_pair(const __half *p) {
+  return __half22float2(*reinterpret_cast<const __half2 *>(p));
+}
+__device__ __forceinline__ float2 stored_pair(const __nv_bfloat16 *p) {
+  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+}
+
+// 36 w_i: an integer times every density deviation of a local reference, added exactly (12 as 8 + 4).
+template <int LAT>
+__device__ __forceinline__ constexpr int weight36(int i) {
+  return LAT == kD3Q19 ? (i == 0 ? 12 : (i < 7 ? 2 : 1)) : (i == 0 ? 16 : (i < 5 ? 4 : 1));
+}
+
+// Densities n_J and, with MOM, momentum sums j_J of the populations arriving at site s (pull), in FP64.
+template <int LAT, class ST, bool MOM>
+__device__ __forceinline__ void arriving_sums(const PopArgs &a, int s, int x, int y, int z, double2 &n,
+                                              double2 (&j)[3]) {
   using L = Lattice<LAT>;
   const ST *buf = static_cast<const ST *>(a.buf);
-  const int64_t N = a.N;
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
-    int x, y, z;
-    coords(s, a.nx, a.ny, x, y, z);
+  int X[3], Y[3], Z[3];
+  axis_offsets<1>(x, a.nx, 1, X);
+  axis_offsets<1>(y, a.ny, a.nx, Y);
+  axis_offsets<1>(z, a.nz, a.nx * a.ny, Z);
+  PairSum<ST> sum, mom[3];
+  PairSum3 ref, rmom[3];
 #pragma unroll
-    for (int J = 0; J < 2; ++J) {
-      double n = 0.0;
+  for (int i = 0; i < L::Q; ++i) {
+    const int src = s + X[1 - L::c(i, 0)] + Y[1 - L::c(i, 1)] + Z[1 - L::c(i, 2)];
+    const auto g = stored_pair(buf + ((int64_t)i * a.N + src) * 2);
+    sum.add(g);
+    if constexpr (MOM) {
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) {
-        const int64_t bwd = site_at(x - L::c(i, 0), y - L::c(i, 1), z - L::c(i, 2), a.nx, a.ny, a.nz);
-        n += pop_value<LAT, ST>(a, buf, i, J, bwd);
+      for (int m = 0; m < L::DIM; ++m) {
+        if (L::c(i, m) > 0) mom[m].add(g);
+        if (L::c(i, m) < 0) mom[m].sub(g);
       }
-      fields[J * N + s] = n;
-      fields[(2 + J) * N + s] = psi_exp ? exp(-1.0 / n) : n;
+    }
+    if constexpr (local_ref<ST>()) {
+      const float2 r = a.nref[src];
+      constexpr float w8 = 8.0f, w4 = 4.0f;
+      const int w = weight36<LAT>(i);
+      if (w == 12) {
+        ref.add(make_float2(w8 * r.x, w8 * r.y));
+        ref.add(make_float2(w4 * r.x, w4 * r.y));
+      } else {
+        const float2 wr = make_float2(float(w) * r.x, float(w) * r.y);
+        ref.add(wr);
+        if constexpr (MOM) {
+#pragma unroll
+          for (int m = 0; m < L::DIM; ++m) {
+            if (L::c(i, m) > 0) rmom[m].add(wr);
+            if (L::c(i, m) < 0) rmom[m].sub(wr);
+          }
+        }
+      }
+    }
+  }
+  const double2 inv = make_double2(a.inv_scale[0][0], a.inv_scale[1][0]), nb = make_double2(a.nbar[0], a.nbar[1]);
+  n = pfma(inv, sum.value(), nb);
+  if constexpr (local_ref<ST>()) n = pfma(pbc(1.0 / 36.0), ref.value(), n);
+  if constexpr (MOM) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      j[m] = m < L::DIM ? pmul(inv, mom[m].value()) : pbc(0.0);
+      if constexpr (local_ref<ST>())
+        if (m < L::DIM) j[m] = pfma(pbc(1.0 / 36.0), rmom[m].value(), j[m]);
     }
   }
 }
 
+// FP64 density fields n_J (and psi_J) from the stored state (pull + sum).
+// fields: [4][N] = n_A, n_B, psi_A, psi_B; psi_J is written only for a component with a self coupling
+// (self bit J): psi enters the force and the pressure times G_JJ only.
+template <int LAT, class ST>
+__global__ void __launch_bounds__(128) fields_kernel(PopArgs a, int psi_exp, int self, double *fields) {
+  const int64_t N = a.N;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < N; q += (int64_t)gridDim.x * blockDim.x) {
+    const int s = (int)q;
+    int x, y, z;
+    a.div.coords(s, a.nx, a.ny, x, y, z);
+    double2 n, j[3];
+    arriving_sums<LAT, ST, false>(a, s, x, y, z, n, j);
+    fields[s] = n.x;
+    fields[N + s] = n.y;
+    if (self & 1) fields[2 * N + s] = psi_exp ? exp(-1.0 / n.x) : n.x;
+    if (self & 2) fields[3 * N + s] = psi_exp ? exp(-1.0 / n.y) : n.y;
+  }
+}
 
-// Eq. sc_force at site s from FP64 fields, +/- pairs first.
-template <int LAT, int STEN>
-__device__ __forceinline__ void force64(const ForceParams &p, const double *fields, int x, int y, int z, int64_t s,
-                                        double F[2][3]) {
-  using SN = Stencil<LAT, STEN>;
-  const double cs2 = 1.0 / 3.0;
-  double S[2][3] = {{0, 0, 0}, {0, 0, 0}}, T[2][3] = {{0, 0, 0}, {0, 0, 0}};
+// Gradient sum_a W v_a f(x + v_a) of an FP64 plane, +/- pairs first.
+template <int STEN_LAT, int STEN>
+__device__ __forceinline__ void gradient64(const double *f, int s, const int *X, const int *Y, const int *Z,
+                                           double (&S)[3]) {
+  using SN = Stencil<STEN_LAT, STEN>;
+  constexpr int H = SN::HALO;
+  S[0] = S[1] = S[2] = 0.0;
 #pragma unroll
   for (int k = 0; k < SN::NH; ++k) {
     const int v0 = SN::v(k, 0), v1 = SN::v(k, 1), v2 = SN::v(k, 2);
-    const int64_t sp = site_at(x + v0, y + v1, z + v2, p.nx, p.ny, p.nz);
-    const int64_t sm = site_at(x - v0, y - v1, z - v2, p.nx, p.ny, p.nz);
-    const double W = SN::W(k);
-    const int v[3] = {v0, v1, v2};
-#pragma unroll
-    for (int J = 0; J < 2; ++J) {
-      const double d = fields[J * p.N + sp] - fields[J * p.N + sm];
-      const double e = fields[(2 + J) * p.N + sp] - fields[(2 + J) * p.N + sm];
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        S[J][m] += W * v[m] * d;
-        T[J][m] += W * v[m] * e;
-      }
-    }
+    const double d = f[s + X[H + v0] + Y[H + v1] + Z[H + v2]] - f[s + X[H - v0] + Y[H - v1] + Z[H - v2]];
+    if (v0) S[0] += SN::W(k) * v0 * d;
+    if (v1) S[1] += SN::W(k) * v1 * d;
+    if (v2) S[2] += SN::W(k) * v2 * d;
   }
-#pragma unroll
-  for (int J = 0; J < 2; ++J)
-#pragma unroll
-    for (int m = 0; m < 3; ++m)
-      F[J][m] = -p.G * cs2 * fields[J * p.N + s] * S[1 - J][m] -
-                p.G_self[J] * cs2 * fields[(2 + J) * p.N + s] * T[J][m];
 }
 
-// Common velocity of Eq. u (force included), FP64 [3][N].
+// Common velocity of Eq. u (force of Eq. sc_force included) at site s, FP64.
 template <int LAT, int STEN, class ST>
-__device__ __forceinline__ void site_velocity(const PopArgs &a, const ForceParams &fp, const double *fields,
-                                              int64_t s, double u[3]) {
-  using L = Lattice<LAT>;
-  const ST *buf = static_cast<const ST *>(a.buf);
+__device__ __forceinline__ void site_velocity(const PopArgs &a, const ForceParams &fp, const double *fields, int s,
+                                              double u[3]) {
+  constexpr int H = Stencil<LAT, STEN>::HALO;
   const int64_t N = a.N;
   int x, y, z;
-  coords(s, a.nx, a.ny, x, y, z);
-  double F[2][3];
-  force64<LAT, STEN>(fp, fields, x, y, z, s, F);
-  double j[2][3] = {{0, 0, 0}, {0, 0, 0}};
+  a.div.coords(s, a.nx, a.ny, x, y, z);
+  double2 n, j[3];
+  arriving_sums<LAT, ST, true>(a, s, x, y, z, n, j);
+  int X[2 * H + 1], Y[2 * H + 1], Z[2 * H + 1];
+  axis_offsets<H>(x, a.nx, 1, X);
+  axis_offsets<H>(y, a.ny, a.nx, Y);
+  axis_offsets<H>(z, a.nz, a.nx * a.ny, Z);
+  const double half_cs2 = 0.5 / 3.0;
+  const double nA = fields[s], nB = fields[N + s];
+  double S[3];
 #pragma unroll
-  for (int J = 0; J < 2; ++J)
+  for (int m = 0; m < 3; ++m) u[m] = j[m].x + j[m].y;
+  // half the force: component A feels the gradient of n_B and the other way round, each its own psi's
+  gradient64<LAT, STEN>(fields, s, X, Y, Z, S);
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      const int64_t bwd = site_at(x - L::c(i, 0), y - L::c(i, 1), z - L::c(i, 2), a.nx, a.ny, a.nz);
-      const double g = pop_value<LAT, ST>(a, buf, i, J, bwd);
+  for (int m = 0; m < 3; ++m) u[m] -= fp.G * half_cs2 * nB * S[m];
+  gradient64<LAT, STEN>(fields + N, s, X, Y, Z, S);
 #pragma unroll
-      for (int m = 0; m < 3; ++m) j[J][m] += L::c(i, m) * g;
-    }
-  const double n = fields[s] + fields[N + s];
+  for (int m = 0; m < 3; ++m) u[m] -= fp.G * half_cs2 * nA * S[m];
 #pragma unroll
-  for (int m = 0; m < 3; ++m) u[m] = ((j[0][m] + 0.5 * F[0][m]) + (j[1][m] + 0.5 * F[1][m])) / n;
+  for (int J = 0; J < 2; ++J) {
+    if (fp.G_self[J] == 0.0) continue;
+    const double *psi = fields + (2 + J) * N;
+    gradient64<LAT, STEN>(psi, s, X, Y, Z, S);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) u[m] -= fp.G_self[J] * half_cs2 * psi[s] * S[m];
+  }
+  const double inv = 1.0 / (nA + nB);
+#pragma unroll
+  for (int m = 0; m < 3; ++m) u[m] *= inv;
 }
 
 template <int LAT, int STEN, class ST>
-__global__ void velocity_kernel(PopArgs a, ForceParams fp, const double *fields, double *u) {
+__global__ void __launch_bounds__(128, 4) velocity_kernel(PopArgs a, ForceParams fp, const double *fields, double *u) {
   const int64_t N = a.N;
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
     double v[3];
-    site_velocity<LAT, STEN, ST>(a, fp, fields, s, v);
+    site_velocity<LAT, STEN, ST>(a, fp, fields, (int)s, v);
 #pragma unroll
     for (int m = 0; m < 3; ++m) u[m * N + s] = v[m];
   }
@@ -209,13 +307,13 @@ __global__ void velocity_kernel(PopArgs a, ForceParams fp, const double *fields,
 // partial sums of sum_alpha |u_alpha(x) - u_prev_alpha(x)| over the sites (fixed
 // grid-stride order, fixed tree); u_prev is overwritten with u.
 template <int LAT, int STEN, class ST>
-__global__ void __launch_bounds__(256) velocity_change_partial_kernel(PopArgs a, ForceParams fp, const double *fields,
+__global__ void __launch_bounds__(256, 2) velocity_change_partial_kernel(PopArgs a, ForceParams fp, const double *fields,
                                                                       double *u_prev, double *partial) {
   const int64_t N = a.N;
   double acc = 0.0;
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
     double v[3];
-    site_velocity<LAT, STEN, ST>(a, fp, fields, s, v);
+    site_velocity<LAT, STEN, ST>(a, fp, fields, (int)s, v);
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       acc += fabs(v[m] - u_prev[m * N + s]);
@@ -234,12 +332,12 @@ __global__ void __launch_bounds__(256) velocity_change_partial_kernel(PopArgs a,
 
 // Centre of mass of one density field's excess over a background value, partial
 // sums (w x, w y, w z, w) with w = n(x) - background, in lattice coordinates.
-__global__ void __launch_bounds__(256) com_partial_kernel(const double *n, int nx, int ny, int64_t N, double bg,
-                                                          double *partial) {
+__global__ void __launch_bounds__(256) com_partial_kernel(const double *n, int nx, int ny, SiteDiv div, int64_t N,
+                                                          double bg, double *partial) {
   double acc[4] = {0, 0, 0, 0};
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
     int x, y, z;
-    coords(s, nx, ny, x, y, z);
+    div.coords((int)s, nx, ny, x, y, z);
     const double w = n[s] - bg;
     acc[0] += w * x;
     acc[1] += w * y;
@@ -261,79 +359,171 @@ __global__ void __launch_bounds__(256) com_partial_kernel(const double *n, int n
     for (int c = 0; c < 4; ++c) partial[blockIdx.x * 4 + c] = red[c][0];
 }
 
-// Block-order finalisation of the two reductions above: kind 0 -> out[0] = scale * sum;
-// kind 1 -> out = (X, Y, Z, M) with M the summed weight and X = sum w x / M.
-__global__ void finalize_measure_kernel(const double *partial, int nblocks, int kind, double scale, double *out) {
-  if (threadIdx.x != 0) return;
-  if (kind == 0) {
-    double acc = 0.0;
-    for (int k = 0; k < nblocks; ++k) acc += partial[k];
-    out[0] = scale * acc;
-    return;
+// Sum of nblocks rows of NC values in a fixed order by one block of 256 threads: a strided sum per thread, then a
+// tree; the sums are returned to thread 0.
+template <int NC>
+__device__ __forceinline__ void block_rows_sum(const double *partial, int nblocks, double (&out)[NC]) {
+  __shared__ double red[NC][256];
+  double acc[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) acc[c] = 0.0;
+  for (int k = threadIdx.x; k < nblocks; k += 256)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] += partial[k * NC + c];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) red[c][threadIdx.x] = acc[c];
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if (threadIdx.x < w)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + w];
+    __syncthreads();
   }
-  double acc[4] = {0, 0, 0, 0};
-  for (int k = 0; k < nblocks; ++k)
-    for (int c = 0; c < 4; ++c) acc[c] += partial[k * 4 + c];
-  out[0] = acc[0] / acc[3];
-  out[1] = acc[1] / acc[3];
-  out[2] = acc[2] / acc[3];
-  out[3] = acc[3];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) out[c] = red[c][0];
 }
 
-// Bulk pressure of Eq. bulkp (e_2 = 1) at one node.
-__global__ void bulk_pressure_kernel(ForceParams fp, const double *fields, int64_t s, double *out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// out[c] = scale * sum of component c of the partial rows (one thread used to add the rows one after another:
+// 63 us for 1024 rows of one component, 230 us of four; 5 and 7 us now).
+template <int NC>
+__global__ void __launch_bounds__(256) finalize_sum_kernel(const double *partial, int nblocks, double scale,
+                                                           double *out) {
+  double s[NC];
+  block_rows_sum<NC>(partial, nblocks, s);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) out[c] = scale * s[c];
+}
+
+// out = (X, Y, Z, M) with M the summed weight and X = sum w x / M.
+__global__ void __launch_bounds__(256) finalize_com_kernel(const double *partial, int nblocks, double *out) {
+  double s[4];
+  block_rows_sum<4>(partial, nblocks, s);
+  if (threadIdx.x == 0) {
+    for (int c = 0; c < 3; ++c) out[c] = s[c] / s[3];
+    out[3] = s[3];
+  }
+}
+
+// Bulk pressure of Eq. bulkp (e_2 = 1) at nodes s0 (out[0]) and, with s1 >= 0, s1 (out[1]).
+__global__ void bulk_pressure_kernel(ForceParams fp, const double *fields, int64_t s0, int64_t s1, double *out) {
+  const int64_t s = threadIdx.x == 0 ? s0 : s1;
+  if (threadIdx.x > 1 || s < 0) return;
   const double cs2 = 1.0 / 3.0;
-  const double nA = fields[s], nB = fields[fp.N + s], psA = fields[2 * fp.N + s], psB = fields[3 * fp.N + s];
-  out[0] = (nA + nB) * cs2 + fp.G * cs2 * nA * nB + 0.5 * fp.G_self[0] * cs2 * psA * psA +
-           0.5 * fp.G_self[1] * cs2 * psB * psB;
+  const double nA = fields[s], nB = fields[fp.N + s];
+  double P = (nA + nB) * cs2 + fp.G * cs2 * nA * nB;
+  for (int J = 0; J < 2; ++J) {
+    if (fp.G_self[J] == 0.0) continue;
+    const double ps = fields[(2 + J) * fp.N + s];
+    P += 0.5 * fp.G_self[J] * cs2 * ps * ps;
+  }
+  out[threadIdx.x] = P;
 }
 
-// sigma[R] minimum (section 3) on one warp; see sc_sigma_minimum in sc.h.
-__global__ void __launch_bounds__(32) sigma_kernel(const double *rows, int nbins, const double *pio, int dim,
-                                                   double R_lo, double R_hi, double R_step, double *out) {
-  const int lane = threadIdx.x;
-  __shared__ double s_C;
-  if (lane == 0) {
-    // trapezoid of r^(dim-1) P_T over the non-empty rows, in order
-    double T = 0.0, rp = 0.0, fp = 0.0, rmax = 0.0;
-    bool first = true;
-    for (int b = 0; b < nbins; ++b) {
-      if (rows[b * 6 + 5] <= 0.0) continue;
-      const double r = rows[b * 6 + 0], pt = rows[b * 6 + 2];
-      const double f = (dim == 3 ? r * r : r) * pt;
-      if (!first) T += 0.5 * (f + fp) * (r - rp);
-      first = false;
-      rp = r;
-      fp = f;
-      rmax = r;
+// sigma[R] minimum (section 3) on one block of 256 threads; see sc_sigma_minimum in sc.h.
+//  * The trapezoid of r^(dim-1) P_T: rows come 256 at a time into shared memory, every thread forms the term of its
+//    row with the last non-empty row before it, and the terms are added in a fixed tree.
+//  * The grid search needs sigma[R] in FP64 only where it can be the minimum: FP32 values of all samples, good to
+//    1e-5 of the sizes of their two terms, leave those whose lower bound is below every upper bound.
+// One warp did both one after another before: 212 us at 128 rows and 6400 samples, now 18 us.
+constexpr int kSigmaThreads = 256;
+__global__ void __launch_bounds__(kSigmaThreads) sigma_kernel(const double *rows, int nbins, const double *pio, int dim,
+                                                              double R_lo, double R_hi, double R_step, double *out) {
+  const int tid = threadIdx.x;
+  __shared__ double s_r[kSigmaThreads], s_f[kSigmaThreads], s_t[kSigmaThreads];
+  __shared__ int s_on[kSigmaThreads];
+  __shared__ int s_i[kSigmaThreads];
+  __shared__ float s_u[kSigmaThreads];
+  double T = 0.0, rp = 0.0, fp = 0.0;  // rp, fp: the last non-empty row of the chunks before
+  bool any = false;
+  for (int b0 = 0; b0 < nbins; b0 += kSigmaThreads) {
+    const int b = b0 + tid;
+    const bool on = b < nbins && rows[b * 6 + 5] > 0.0;
+    const double r = on ? rows[b * 6 + 0] : 0.0, pt = on ? rows[b * 6 + 2] : 0.0;
+    const double f = (dim == 3 ? r * r : r) * pt;
+    s_on[tid] = on;
+    s_r[tid] = r;
+    s_f[tid] = f;
+    __syncthreads();
+    double term = 0.0;
+    if (on) {
+      int q = tid - 1;
+      while (q >= 0 && !s_on[q]) --q;
+      if (q >= 0)
+        term = 0.5 * (f + s_f[q]) * (r - s_r[q]);
+      else if (any)
+        term = 0.5 * (f + fp) * (r - rp);
     }
-    const double Pout = pio[1];
-    s_C = Pout * (dim == 3 ? rmax * rmax * rmax / 3.0 : rmax * rmax / 2.0) - T;
+    s_t[tid] = term;
+    int last = kSigmaThreads - 1;
+    while (last >= 0 && !s_on[last]) --last;
+    if (last >= 0) {
+      rp = s_r[last];
+      fp = s_f[last];
+      any = true;
+    }
+    __syncthreads();
+    for (int w = kSigmaThreads / 2; w > 0; w >>= 1) {
+      if (tid < w) s_t[tid] += s_t[tid + w];
+      __syncthreads();
+    }
+    T += s_t[0];
+    __syncthreads();
   }
-  __syncwarp();
-  const double Pin = pio[0], Pout = pio[1], dP = Pin - Pout, C = s_C;
+  const double Pin = pio[0], Pout = pio[1], dP = Pin - Pout;
+  const double C = Pout * (dim == 3 ? rp * rp * rp / 3.0 : rp * rp / 2.0) - T;
   auto sigma = [&](double R) { return dim == 3 ? dP * R / 3.0 + C / (R * R) : dP * R / 2.0 + C / R; };
-  // grid search: each lane scans a strided subset, then a warp argmin (lowest index on ties)
+  // the grid: lowest index on ties
   const int ng = int(floor((R_hi - R_lo) / R_step + 0.5)) + 1;
+  const float c1 = float(dim == 3 ? dP / 3.0 : dP / 2.0), c2 = float(C), lo = float(R_lo), st = float(R_step);
+  auto bounds = [&](int k, float &down, float &up) {
+    const float R = fmaf(float(k), st, lo), u = c1 * R, v = dim == 3 ? c2 / (R * R) : c2 / R, m = 1e-5f * (fabsf(u) + fabsf(v));
+    down = u + v - m;
+    up = u + v + m;
+  };
+  float best_up = INFINITY;
+  for (int k = tid; k < ng; k += kSigmaThreads) {
+    float down, up;
+    bounds(k, down, up);
+    best_up = fminf(best_up, up);  // a NaN bound is ignored here and its sample kept below
+  }
+  s_u[tid] = best_up;
+  __syncthreads();
+  for (int w = kSigmaThreads / 2; w > 0; w >>= 1) {
+    if (tid < w) s_u[tid] = fminf(s_u[tid], s_u[tid + w]);
+    __syncthreads();
+  }
+  // sizes outside FP32's comfortable range: every sample in FP64
+  const double big = fmax(fabs(dP), fabs(C)), small = fmin(fabs(dP), fabs(C));
+  best_up = (big < 1e25 && small > 1e-25 && R_lo > 1e-4 && R_hi < 1e8) ? s_u[0] : INFINITY;
   double best = INFINITY;
   int bi = -1;
-  for (int k = lane; k < ng; k += 32) {
+  for (int k = tid; k < ng; k += kSigmaThreads) {
+    float down, up;
+    bounds(k, down, up);
+    if (down > best_up && down < INFINITY) continue;
     const double v = sigma(R_lo + k * R_step);
     if (v < best) {
       best = v;
       bi = k;
     }
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    const double ob = __shfl_down_sync(0xffffffffu, best, off);
-    const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-    if (oi >= 0 && (ob < best || (ob == best && (bi < 0 || oi < bi)))) {
-      best = ob;
-      bi = oi;
+  s_t[tid] = best;
+  s_i[tid] = bi;
+  __syncthreads();
+  for (int w = kSigmaThreads / 2; w > 0; w >>= 1) {
+    if (tid < w) {
+      const double ob = s_t[tid + w];
+      const int oi = s_i[tid + w];
+      if (oi >= 0 && (ob < s_t[tid] || (ob == s_t[tid] && (s_i[tid] < 0 || oi < s_i[tid])))) {
+        s_t[tid] = ob;
+        s_i[tid] = oi;
+      }
     }
+    __syncthreads();
   }
-  if (lane == 0) {
+  if (tid == 0) {
+    bi = s_i[0];
     const double Rs = dim == 3 ? cbrt(6.0 * C / dP) : sqrt(2.0 * C / dP);
     out[0] = dP;
     out[1] = C;
@@ -439,8 +629,20 @@ __global__ void curvature_fit_kernel(const double *Rs, const double *sig, int n,
   out[3] = sqrt(rss / n);
 }
 
+// FP32 value as FP64 by integer arithmetic: the conversion instruction issues at the FP64 rate, 1/64 of this.
+// Zeros, denormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v), e = b & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) return (double)v;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
 // Deterministic FP64 totals: per-block partial sums (fixed grid-stride order,
 // fixed tree) of mass_A, mass_B and momentum; finalised in block order.
+// The total momentum is a small difference of large sums, so its terms are FP64 populations added one by one.
+// FP64-bound: 142 FP64 instructions a site (conversions in integers, no product with a scale of one, no zero
+// terms) against 304 before: 128^3 BF16 987 -> 757 us.
 template <int LAT, class ST>
 __global__ void __launch_bounds__(256) totals_partial_kernel(PopArgs a, double *partial) {
   using L = Lattice<LAT>;
@@ -448,16 +650,31 @@ __global__ void __launch_bounds__(256) totals_partial_kernel(PopArgs a, double *
   const int64_t N = a.N;
   double acc[5] = {0, 0, 0, 0, 0};
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
+    float2 nref = make_float2(0.0f, 0.0f);
+    if constexpr (local_ref<ST>()) nref = a.nref[s];
+    double g[2][L::Q];
 #pragma unroll
-    for (int J = 0; J < 2; ++J)
+    for (int i = 0; i < L::Q; ++i) {
+      // stored at the collision site: sums over all sites need no pull
+      const auto v = stored_pair(buf + ((int64_t)i * N + s) * 2);
+      g[0][i] = widen(v.x);
+      g[1][i] = widen(v.y);
+    }
+#pragma unroll
+    for (int J = 0; J < 2; ++J) {
+      const double ref = a.nbar[J] + (local_ref<ST>() ? widen(J == 0 ? nref.x : nref.y) : 0.0);
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) {
-        // stored at the collision site: sums over all sites need no pull
-        const double f = pop_value<LAT, ST>(a, buf, i, J, s);
+        const double wr = __dmul_rn(L::w(i), ref);
+        const double f = scaled_units<ST>() ? __fma_rn(g[J][i], a.inv_scale[J][0], wr) : __dadd_rn(g[J][i], wr);
         acc[J] += f;
 #pragma unroll
-        for (int m = 0; m < 3; ++m) acc[2 + m] += L::c(i, m) * f;
+        for (int m = 0; m < 3; ++m) {
+          if (L::c(i, m) > 0) acc[2 + m] += f;
+          if (L::c(i, m) < 0) acc[2 + m] -= f;
+        }
       }
+    }
   }
   __shared__ double red[5][256];
 #pragma unroll
@@ -472,12 +689,24 @@ __global__ void __launch_bounds__(256) totals_partial_kernel(PopArgs a, double *
   if (threadIdx.x < 5) partial[blockIdx.x * 5 + threadIdx.x] = red[threadIdx.x][0];
 }
 
-__global__ void totals_finalize_kernel(const double *partial, int nblocks, int ncomp, double *out) {
-  const int c = threadIdx.x;
-  if (c >= ncomp) return;
+// Sums of the NC components of nblocks rows added in block order (the mean densities and the totals keep this
+// order: the first fix the stored bits of every population, the others are differences).  The rows come into
+// shared memory by all threads; one thread per component adds them.
+template <int NC>
+__global__ void __launch_bounds__(256) totals_finalize_kernel(const double *partial, int nblocks, double *out) {
+  __shared__ double rows[256 * NC];
   double acc = 0.0;
-  for (int k = 0; k < nblocks; ++k) acc += partial[k * ncomp + c];
-  out[c] = acc;
+  for (int k0 = 0; k0 < nblocks; k0 += 256) {
+    const int n = min(256, nblocks - k0) * NC;
+    for (int k = threadIdx.x; k < n; k += 256) rows[k] = partial[k0 * NC + k];
+    __syncthreads();
+    if (threadIdx.x < NC) {
+#pragma unroll 8
+      for (int k = threadIdx.x; k < n; k += NC) acc += rows[k];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < NC) out[threadIdx.x] = acc;
 }
 
 // Deterministic FP64 sums of two fields (used for the mean initial densities).

@@ -260,6 +260,26 @@ __host__ __device__ constexpr bool local_ref() {
   return sizeof(ST) == 2;
 }
 
+// Exact quotient of 0 <= n < 2^31 by a fixed divisor: mul = ceil(2^(32 + shift) / div), shift =
+// ceil(log2 div) - 1, so that the rounding of mul adds less than 1 / div to n / div.
+struct FastDiv {
+  unsigned mul, shift, div;
+  __host__ __device__ __forceinline__ unsigned quot(unsigned n) const {
+    return div == 1 ? n : (unsigned)(((unsigned long long)n * mul) >> 32) >> shift;
+  }
+};
+
+// Coordinates of site s < 2^31 by two fixed-divisor quotients.
+struct SiteDiv {
+  FastDiv dx, dy;
+  __device__ __forceinline__ void coords(int s, int nx, int ny, int &x, int &y, int &z) const {
+    const unsigned q = dx.quot((unsigned)s);
+    x = s - (int)q * nx;
+    z = (int)dy.quot(q);
+    y = (int)q - z * ny;
+  }
+};
+
 __host__ __device__ __forceinline__ int wrapi(int a, int n) {
   // a in [-n, 2n)
   return a < 0 ? a + n : (a >= n ? a - n : a);

@@ -23,4 +23,8 @@ sc_status validate_profile_request(const sc_params *p, int32_t kind, const doubl
 // ProfileArgs of a validated request (chunk set by the launcher).
 ProfileArgs profile_args(const sc_params *p, int32_t kind, const double centre[3], double bin_width, int32_t nbins);
 
+// Fixed-divisor quotients (FastDiv) of the lattice sides.
+FastDiv fast_div(unsigned d);
+SiteDiv site_div(const sc_params *p);
+
 }  // namespace scgb

@@ -77,6 +77,7 @@ extern "C" sc_status sc_pressure_profile_noalloc(const sc_params *p, const doubl
   fp.ny = p->ny;
   fp.nz = p->nz;
   fp.N = (int64_t)p->nx * p->ny * p->nz;
+  fp.div = site_div(p);
   // as many blocks as the scratch holds rows for (at most kMaxBlocks, at least one)
   const cudaError_t e = launch_profile(p->lattice, p->stencil, fp, profile_args(p, kind, centre, bin_width, nbins),
                                        DensityFields{nA, nB, p->psi_self == SC_PSI_EXP ? 1 : 0}, scratch,

@@ -22,21 +22,12 @@
 
 namespace scgb {
 
-// Exact quotient of 0 <= n < 2^31 by a fixed divisor: mul = ceil(2^(32 + shift) / div), shift =
-// ceil(log2 div) - 1, so that the rounding of mul adds less than 1 / div to n / div.
-struct FastDiv {
-  unsigned mul, shift, div;
-  __host__ __device__ __forceinline__ unsigned quot(unsigned n) const {
-    return div == 1 ? n : (unsigned)(((unsigned long long)n * mul) >> 32) >> shift;
-  }
-};
-
 // One lattice as the two passes step it.
 template <class CT>
 struct SplitArgs {
   StepArgs<CT> a;
   P2<CT> *mom;  // [4 or 5][N]: density deviation, momentum sums x, y, z, with a self coupling psi deviation
-  FastDiv dx, dy;
+  SiteDiv div;
 };
 
 // Launches follow one another as programmatic dependents: a pass starts while the one before drains, and
@@ -49,21 +40,13 @@ __device__ __forceinline__ void pass_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-template <class CT>
-__device__ __forceinline__ void split_coords(const SplitArgs<CT> &m, int s, int &x, int &y, int &z) {
-  const unsigned q = m.dx.quot((unsigned)s);
-  x = s - (int)q * m.a.nx;
-  z = (int)m.dy.quot(q);
-  y = (int)q - z * m.a.ny;
-}
-
 // Moments pass at site s.
 template <class ST, class CT>
 __device__ __forceinline__ void split_moments(const SplitArgs<CT> &m, const ST *src, const float2 *nsrc, int s) {
   using L = Lattice<kD3Q19>;
   const StepArgs<CT> &a = m.a;
   int x, y, z;
-  split_coords<CT>(m, s, x, y, z);
+  m.div.coords(s, a.nx, a.ny, x, y, z);
   // site offset of the source for a velocity component of -1, 0, +1
   const int W = a.nx * a.ny;
   const int X[3] = {x == a.nx - 1 ? 1 - a.nx : 1, 0, x == 0 ? a.nx - 1 : -1};
@@ -100,7 +83,7 @@ __device__ __forceinline__ void split_collide(const SplitArgs<CT> &m, ST *dst, f
   constexpr int H = SN::HALO;
   const StepArgs<CT> &a = m.a;
   int x, y, z;
-  split_coords<CT>(m, s, x, y, z);
+  m.div.coords(s, a.nx, a.ny, x, y, z);
   const P2<CT> *dnp = m.mom, *psp = m.mom + 4 * a.N;
   const P2<CT> j[3] = {m.mom[a.N + s], m.mom[2 * a.N + s], m.mom[3 * a.N + s]};
   const P2<CT> dn = dnp[s];
