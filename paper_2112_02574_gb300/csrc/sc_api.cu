@@ -112,7 +112,9 @@ int default_tile_z(const sc_params *p) {
 
 // The two-pass step can serve these parameters.
 bool split_eligible(const sc_params *p) {
-  return p->lattice == SC_D3Q19 && tau_one(p) && p->nx >= 4 && p->ny >= 4 && p->nz >= 4;
+  if (p->lattice != SC_D3Q19 || !tau_one(p) || p->nx < 4 || p->ny < 4 || p->nz < 4) return false;
+  // its byte offsets within one direction are 32 bits: at most 16 (FP64) or 8 bytes a site
+  return (int64_t)p->nx * p->ny * p->nz <= (int64_t(1) << 32) / (p->storage == SC_STORE_F64 ? 16 : 8);
 }
 // ... and does: the step kernel is left to the library (no variant, tile or pipeline asked for), and either
 // the lattice cannot take the staged kernel, or it is FP64 (no density is summed twice), or the moments stay

@@ -89,6 +89,13 @@ __device__ __forceinline__ void store_hint(double2 *p, double2 v, unsigned long 
   asm volatile("st.global.L2::cache_hint.v2.f64 [%0], {%1, %2}, %3;" ::"l"(p), "d"(v.x), "d"(v.y), "l"(pol) : "memory");
 }
 
+// Element at a byte offset below 2^32 from a pointer that is the same for every thread: the address is the
+// uniform base plus a 32-bit register, without 64-bit arithmetic per access.
+template <class T>
+__device__ __forceinline__ T *at(T *base, unsigned bytes) {
+  return reinterpret_cast<T *>(reinterpret_cast<uintptr_t>(base) + bytes);
+}
+
 // Moments pass at site s.
 template <class ST, class CT>
 __device__ __forceinline__ void split_moments(const SplitArgs<CT> &m, const ST *src, const float2 *nsrc, int s) {
@@ -97,18 +104,21 @@ __device__ __forceinline__ void split_moments(const SplitArgs<CT> &m, const ST *
   const L2Policy pol(m.keep_moments);
   int x, y, z;
   m.div.coords(s, a.nx, a.ny, x, y, z);
-  // site offset of the source for a velocity component of -1, 0, +1
+  // byte offset of the source for a velocity component of -1, 0, +1
+  constexpr int E = 2 * sizeof(ST);
   const int W = a.nx * a.ny;
-  const int X[3] = {x == a.nx - 1 ? 1 - a.nx : 1, 0, x == 0 ? a.nx - 1 : -1};
-  const int Y[3] = {y == a.ny - 1 ? a.nx * (1 - a.ny) : a.nx, 0, y == 0 ? a.nx * (a.ny - 1) : -a.nx};
-  const int Z[3] = {z == a.nz - 1 ? W * (1 - a.nz) : W, 0, z == 0 ? W * (a.nz - 1) : -W};
+  const unsigned X[3] = {unsigned(x == a.nx - 1 ? 1 - a.nx : 1) * E, 0u, unsigned(x == 0 ? a.nx - 1 : -1) * E};
+  const unsigned Y[3] = {unsigned(y == a.ny - 1 ? a.nx * (1 - a.ny) : a.nx) * E, 0u,
+                         unsigned(y == 0 ? a.nx * (a.ny - 1) : -a.nx) * E};
+  const unsigned Z[3] = {unsigned(z == a.nz - 1 ? W * (1 - a.nz) : W) * E, 0u,
+                         unsigned(z == 0 ? W * (a.nz - 1) : -W) * E};
   P2<CT> g[L::Q];
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
-    const int site = s + X[L::c(i, 0) + 1] + Y[L::c(i, 1) + 1] + Z[L::c(i, 2) + 1];
-    g[i] = load_hint(src + ((int64_t)i * a.N + site) * 2, pol.first);
+    const unsigned o = unsigned(s) * E + X[L::c(i, 0) + 1] + Y[L::c(i, 1) + 1] + Z[L::c(i, 2) + 1];
+    g[i] = load_hint(at(src + (int64_t)i * a.N * 2, o), pol.first);
     if constexpr (local_ref<ST>()) {
-      const float2 ns = nsrc[site];
+      const float2 ns = *at(nsrc, o * (8 / E));
       g[i] = pfma(wpair<kD3Q19, ST, CT>(i, a.scale), pset(CT(ns.x), CT(ns.y)), g[i]);
     }
   }
@@ -118,12 +128,13 @@ __device__ __forceinline__ void split_moments(const SplitArgs<CT> &m, const ST *
   const P2<CT> dn = unscale<ST, CT>(sum, a.inv_scale);
   P2<CT> j[3];
   momentum_sums<kD3Q19, CT>(g, j);
-  store_hint(m.mom + s, dn, pol.last);
-  store_hint(m.mom + a.N + s, j[0], pol.last);
-  store_hint(m.mom + 2 * a.N + s, j[1], pol.last);
-  store_hint(m.mom + 3 * a.N + s, j[2], pol.last);
+  const unsigned p = unsigned(s) * unsigned(sizeof(P2<CT>));
+  store_hint(at(m.mom, p), dn, pol.last);
+  store_hint(at(m.mom + a.N, p), j[0], pol.last);
+  store_hint(at(m.mom + 2 * a.N, p), j[1], pol.last);
+  store_hint(at(m.mom + 3 * a.N, p), j[2], pol.last);
   if (a.self_on)
-    store_hint(m.mom + 4 * a.N + s, psi_deviation<CT>(dn, a.nbar, a.psibar, a.psi_exp, a.gself), pol.last);
+    store_hint(at(m.mom + 4 * a.N, p), psi_deviation<CT>(dn, a.nbar, a.psibar, a.psi_exp, a.gself), pol.last);
 }
 
 // Collision pass at site s: Eq. sc_force from the stored densities in force_pair's order, then the shared collision.
@@ -136,37 +147,39 @@ __device__ __forceinline__ void split_collide(const SplitArgs<CT> &m, ST *dst, f
   const L2Policy pol(m.keep_moments);
   int x, y, z;
   m.div.coords(s, a.nx, a.ny, x, y, z);
+  constexpr int E = sizeof(P2<CT>);
+  const unsigned o = unsigned(s) * E;
   const P2<CT> *dnp = m.mom, *psp = m.mom + 4 * a.N;
-  const CT *jp = reinterpret_cast<const CT *>(m.mom + s);
-  const P2<CT> j[3] = {load_hint(jp + 2 * a.N, pol.first), load_hint(jp + 4 * a.N, pol.first),
-                       load_hint(jp + 6 * a.N, pol.first)};
-  const P2<CT> dn = dnp[s];
+  const CT *jp = reinterpret_cast<const CT *>(m.mom);
+  const P2<CT> j[3] = {load_hint(at(jp + 2 * a.N, o), pol.first), load_hint(at(jp + 4 * a.N, o), pol.first),
+                       load_hint(at(jp + 6 * a.N, o), pol.first)};
+  const P2<CT> dn = *at(dnp, o);
   const P2<CT> n = padd(a.nbar, dn);
-  int X[2 * H + 1], Y[2 * H + 1], Z[2 * H + 1];
+  unsigned X[2 * H + 1], Y[2 * H + 1], Z[2 * H + 1];  // byte offsets
   const int W = a.nx * a.ny;
 #pragma unroll
   for (int d = -H; d <= H; ++d) {
-    X[d + H] = wrapi(x + d, a.nx) - x;
-    Y[d + H] = (wrapi(y + d, a.ny) - y) * a.nx;
-    Z[d + H] = (wrapi(z + d, a.nz) - z) * W;
+    X[d + H] = unsigned(wrapi(x + d, a.nx) - x) * E;
+    Y[d + H] = unsigned((wrapi(y + d, a.ny) - y) * a.nx) * E;
+    Z[d + H] = unsigned((wrapi(z + d, a.nz) - z) * W) * E;
   }
   P2<CT> S[3] = {pbc(CT(0)), pbc(CT(0)), pbc(CT(0))}, T[3] = {pbc(CT(0)), pbc(CT(0)), pbc(CT(0))};
 #pragma unroll
   for (int k = 0; k < SN::NH; ++k) {
     const int vx = SN::v(k, 0), vy = SN::v(k, 1), vz = SN::v(k, 2);
-    const int ip = s + X[H + vx] + Y[H + vy] + Z[H + vz], im = s + X[H - vx] + Y[H - vy] + Z[H - vz];
-    const P2<CT> d = psub(dnp[ip], dnp[im]);
+    const unsigned ip = o + X[H + vx] + Y[H + vy] + Z[H + vz], im = o + X[H - vx] + Y[H - vy] + Z[H - vz];
+    const P2<CT> d = psub(*at(dnp, ip), *at(dnp, im));
     if (vx) S[0] = pfma(pbc(CT(SN::W(k) * vx)), d, S[0]);
     if (vy) S[1] = pfma(pbc(CT(SN::W(k) * vy)), d, S[1]);
     if (vz) S[2] = pfma(pbc(CT(SN::W(k) * vz)), d, S[2]);
     if (a.self_on) {
-      const P2<CT> e = psub(psp[ip], psp[im]);
+      const P2<CT> e = psub(*at(psp, ip), *at(psp, im));
       if (vx) T[0] = pfma(pbc(CT(SN::W(k) * vx)), e, T[0]);
       if (vy) T[1] = pfma(pbc(CT(SN::W(k) * vy)), e, T[1]);
       if (vz) T[2] = pfma(pbc(CT(SN::W(k) * vz)), e, T[2]);
     }
   }
-  const P2<CT> psi = a.self_on ? padd(a.psibar, psp[s]) : pbc(CT(0));
+  const P2<CT> psi = a.self_on ? padd(a.psibar, *at(psp, o)) : pbc(CT(0));
   const P2<CT> cn = pmul(pbc(a.gcross), n), cp = pmul(a.gself, psi);
   P2<CT> F[3], h[3], out[L::Q];
 #pragma unroll
@@ -177,8 +190,9 @@ __device__ __forceinline__ void split_collide(const SplitArgs<CT> &m, ST *dst, f
   collide_pair<kD3Q19, ST, CT, true>(a, nullptr, n, dn, u, F, out);
   check_density<CT>(a, n);
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) Codec2<ST, CT>::store(dst + ((int64_t)i * a.N + s) * 2, out[i], a.scale);
-  if constexpr (local_ref<ST>()) ndst[s] = make_float2(float(dn.x), float(dn.y));
+  for (int i = 0; i < L::Q; ++i)
+    Codec2<ST, CT>::store(at(dst + (int64_t)i * a.N * 2, unsigned(s) * unsigned(2 * sizeof(ST))), out[i], a.scale);
+  if constexpr (local_ref<ST>()) *at(ndst, unsigned(s) * 8u) = make_float2(float(dn.x), float(dn.y));
 }
 
 // Threads per block and the blocks per SM the register allocation must allow (64 registers a thread, 80 for
