@@ -164,7 +164,7 @@ struct Stencil<kD3Q19, kE6> {
 // deviations high in the normal range (a power of two changes no rounding of a
 // normal FP16 number, only how far the values sit from underflow and overflow);
 // BF16 has the FP32 exponent range and needs none.  SMEM selects plain loads
-// (shared memory) instead of read-only-cache loads (global memory).
+// (shared memory, or global memory that the launch before may still be writing) instead of read-only-cache loads.
 template <class ST, class CT>
 struct Codec2;
 template <>
@@ -283,6 +283,16 @@ struct SiteDiv {
 __host__ __device__ __forceinline__ int wrapi(int a, int n) {
   // a in [-n, 2n)
   return a < 0 ? a + n : (a >= n ? a - n : a);
+}
+
+// The two-pass and the D2Q9 step kernels follow one another as programmatic dependents: a kernel starts while the
+// one before drains, and waits here before its first access to what that one wrote.  The launch of the next kernel
+// is allowed only after the wait, so that at most two are on the device and none starts (and caches lines in L1)
+// before the last but one is complete; they load no population or moment through the read-only path, whose data
+// must not change while a kernel runs.
+__device__ __forceinline__ void pass_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 }  // namespace scgb

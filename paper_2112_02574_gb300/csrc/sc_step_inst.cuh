@@ -27,6 +27,25 @@ inline bool attr_once(const void *k, size_t smem) {
   return true;
 }
 
+// A launch that may start while the launch before it in the stream drains (see pass_begin).  For D2Q9 the launch
+// latency is a good part of a step: 64^2 FP32 2.09 -> 1.79 us a step of a replayed graph, 256^2 3.18 -> 2.93.  The
+// one-pass D3Q19 kernels keep plain launches: they lose (97^3 FP32 with tau = 0.9 90.7 -> 96.3 us, staged FP16 160^3
+// 176 -> 182: blocks of the next step take slots and wait while this one still has blocks to place).
+template <class... P, class... A>
+cudaError_t launch_pass(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 // T1 selects the tau_A = tau_B = 1 instantiation (StepArgs::tau_one).
 template <int LAT, int STEN, class ST, class CT, int TY>
 cudaError_t launch_one(const StepLaunch &l, const StepArgs<CT> &a) {
@@ -34,6 +53,7 @@ cudaError_t launch_one(const StepLaunch &l, const StepArgs<CT> &a) {
   auto *k = a.tau_one ? sc_step_kernel<LAT, STEN, ST, CT, TY, true> : sc_step_kernel<LAT, STEN, ST, CT, TY, false>;
   if (!attr_once(reinterpret_cast<const void *>(k), smem)) return cudaGetLastError();
   const dim3 grid = a.zbal_k > 0 ? dim3(a.zbal_k * a.zbal_cols + a.zbal_rem) : l.grid;
+  if constexpr (LAT == kD2Q9) return launch_pass(k, grid, dim3(32, TY), smem, l.stream, a);
   k<<<grid, dim3(32, TY), smem, l.stream>>>(a);
   return cudaGetLastError();
 }

@@ -58,9 +58,10 @@ __device__ __forceinline__ P2<CT> pull_site(const ST *__restrict__ src, int gx, 
   for (int i = 0; i < L::Q; ++i) {
     const int cx = L::c(i, 0), cy = L::c(i, 1), cz = L::c(i, 2);
     const int site = X[cx + 1] + nx * (Y[cy + 1] + ny * Z[cz + 1]);
-    P2<CT> g = Codec2<ST, CT>::template load<false>(src + ((int64_t)i * N + site) * 2, inv_scale);
+    // D2Q9 launches are programmatic dependents (see pass_begin): plain loads
+    P2<CT> g = Codec2<ST, CT>::template load<LAT == kD2Q9>(src + ((int64_t)i * N + site) * 2, inv_scale);
     if constexpr (local_ref<ST>()) {
-      const float2 ns = __ldg(nsrc + site);
+      const float2 ns = LAT == kD2Q9 ? nsrc[site] : __ldg(nsrc + site);
       g = pfma(wpair<LAT, ST, CT>(i, scale), pset(CT(ns.x), CT(ns.y)), g);
     }
     if (V) v[i] = g;
@@ -527,6 +528,7 @@ __global__ void __launch_bounds__(32 * TY, (TY >= 16 ? 1 : 16 / TY)) sc_step_ker
   int bx, by, z0, zend;
   bool down;
   block_work(a, bx, by, z0, zend, down);
+  if constexpr (LAT == kD2Q9) pass_begin();
   step_block<LAT, STEN, ST, CT, TY, T1>(a, bx, by, z0, zend, down, smem_raw);
 }
 

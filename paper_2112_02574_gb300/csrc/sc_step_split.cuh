@@ -31,16 +31,6 @@ struct SplitArgs {
   SiteDiv div;
 };
 
-// Launches follow one another as programmatic dependents: a pass starts while the one before drains, and
-// waits here before its first access to what that one wrote.  The launch of the next pass is allowed only
-// after the wait, so that at most two passes are on the device and no pass starts (and caches lines in L1)
-// before the last but one is complete; no load goes through the read-only path, whose data must not change
-// while a kernel runs.
-__device__ __forceinline__ void pass_begin() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // L2 eviction priorities.  The moments are written by one pass and read by the next; the populations of a large
 // lattice stream through L2 in between and would push them out, though the next step cannot find them there
 // either.  Where the moments fit in L2 (keep_moments) they are written with evict-last, the populations are read
