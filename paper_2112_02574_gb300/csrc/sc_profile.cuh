@@ -59,7 +59,7 @@ struct DensityFields {
 
 // Weighted sums of the interaction part of the pressure tensor (Eq. sm:pt) at one site: over the stencil pairs +/- v,
 //   t(v) = c_s^2/2 { G [n_A(x) n_B(+/-v) + n_B(x) n_A(+/-v)] + sum_J G_JJ psi_J(x) psi_J(+/-v) },  f(+/-v) = f(x+v) + f(x-v),
-// visit(v, W t(v)) is called for each; P_mu,nu = c_s^2 (n_A + n_B) delta + sum W t v_mu v_nu.  psi is read only for a
+// visit(v, t(v)) is called for each (W left to the caller: it is one factor per shell |v|^2); P_mu,nu = c_s^2 (n_A + n_B) delta + sum W t v_mu v_nu.  psi is read only for a
 // component with a self coupling.
 template <int LAT, int STEN, class FA, class F>
 __device__ __forceinline__ void ptensor_terms(const ForceParams &p, const FA &fld, int x, int y, int z, int s, double nA,
@@ -81,7 +81,7 @@ __device__ __forceinline__ void ptensor_terms(const ForceParams &p, const FA &fl
     double t = qA * (fld(0, sp) + fld(0, sm)) + qB * (fld(1, sp) + fld(1, sm));
     if (sA) t += pA * (fld(2, sp) + fld(2, sm));
     if (sB) t += pB * (fld(3, sp) + fld(3, sm));
-    visit(k, SN::W(k) * t);
+    visit(k, t);
   }
 }
 
@@ -112,7 +112,7 @@ __device__ __forceinline__ double min_image(int c, double centre, int L) {
 // needs P_N = e.P.e and the trace, two sums over the stencil pairs (Eq. pt_projection with (v.d)^2 / r^2); sites
 // outside the last shell stop at their r^2; the distances to the centre come from a table per axis; four sites are
 // added to the bins at a time (24 lanes) unless two of them share a bin.  Several warps a block keep the FP64 pipe
-// busy.  Radial profile of 128^3 with 128 bins: 1190 -> 585 us, its
+// busy.  Radial profile of 128^3 with 128 bins: 1190 -> 550 us, its
 // finalisation (one thread per bin before) 500 -> 10 us.
 template <int LAT, int STEN, int KIND, class FA>
 __global__ void __launch_bounds__(256) profile_partial_kernel(ForceParams fp, ProfileArgs pa, FA fld, int tables,
@@ -170,21 +170,43 @@ __global__ void __launch_bounds__(256) profile_partial_kernel(ForceParams fp, Pr
       if (bin >= pa.nbins) bin = -1;
       if (bin >= 0) {
         const double nA = fld(0, s), nB = fld(1, s), ideal = (nA + nB) * (1.0 / 3.0);
-        double sN = 0.0, sT = 0.0;  // P_N's sum; the trace's (radial) or P_T's
+        // P_N's sum; the trace's (radial) or P_T's: per shell, then weighted
+        double shN[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, shT[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, sN = 0.0, sT = 0.0;
         ptensor_terms<LAT, STEN>(fp, fld, x, y, z, s, nA, nB, [&](int k, double t) {
-          const int v0 = SN::v(k, 0), v1 = SN::v(k, 1), v2 = SN::v(k, 2);
+          const int v0 = SN::v(k, 0), v1 = SN::v(k, 1), v2 = SN::v(k, 2), sh = v0 * v0 + v1 * v1 + v2 * v2;
           if constexpr (RADIAL) {
-            const double q = v0 * d0 + v1 * d1 + v2 * d2;
-            sN += q * q * t;
-            sT += (pa.dim == 3 ? double(v0 * v0 + v1 * v1 + v2 * v2) : double(v0 * v0 + v1 * v1)) * t;
+            // v.d without the terms of a zero component
+            const double a0 = v0 < 0 ? -d0 : d0, a1 = v1 < 0 ? -d1 : d1, a2 = v2 < 0 ? -d2 : d2;
+            double q = v0 ? a0 : (v1 ? a1 : a2);
+            if (v0 && v1) q += a1;
+            if ((v0 || v1) && v2) q += a2;
+            if (sh == 4) q *= 2.0;  // (2, 0, 0)
+            shN[sh] += q * q * t;
+            if (pa.dim == 3 || v2 == 0)
+              shT[sh] += t;
+            else
+              shT[0] += SN::W(k) * (v0 * v0 + v1 * v1) * t;  // two dimensions: the trace has no zz
           } else if constexpr (KIND == SC_PROFILE_PLANAR_Z) {
-            if (v2) sN += double(v2 * v2) * t;
-            if (v0 || v1) sT += double(v0 * v0 + v1 * v1) * t;
+            if (v2) sN += SN::W(k) * (v2 * v2) * t;
+            if (v0 || v1) sT += SN::W(k) * (v0 * v0 + v1 * v1) * t;
           } else {
-            if (v0) sN += double(v0 * v0) * t;
-            if (v1) sT += double(v1 * v1) * t;
+            if (v0) sN += SN::W(k) * (v0 * v0) * t;
+            if (v1) sT += SN::W(k) * (v1 * v1) * t;
           }
         });
+        if constexpr (RADIAL) {
+          sT = shT[0];
+#pragma unroll
+          for (int sh = 1; sh <= 4; ++sh) {
+            double W = 0.0;
+#pragma unroll
+            for (int k = 0; k < SN::NH; ++k)
+              if (SN::v(k, 0) * SN::v(k, 0) + SN::v(k, 1) * SN::v(k, 1) + SN::v(k, 2) * SN::v(k, 2) == sh) W = SN::W(k);
+            if (W == 0.0) continue;  // no such shell
+            sN += W * shN[sh];
+            sT += W * sh * shT[sh];
+          }
+        }
         double PN, PT;
         if constexpr (RADIAL) {
           const double tr = pa.dim * ideal + sT;
