@@ -119,14 +119,16 @@ int default_tile_z(const sc_params *p) {
 // The two-pass step can serve these parameters.
 bool split_eligible(const sc_params *p) {
   if (p->lattice != SC_D3Q19 || !tau_one(p) || p->nx < 4 || p->ny < 4 || p->nz < 4) return false;
-  // its byte offsets within one direction are 32 bits: at most 16 (FP64) or 8 bytes a site
-  return (int64_t)p->nx * p->ny * p->nz <= (int64_t(1) << 32) / (p->storage == SC_STORE_F64 ? 16 : 8);
+  // its byte offsets within one direction are 32 bits: at most 8 bytes a site (16 in FP64; twice that with psi)
+  const int64_t site = (p->storage == SC_STORE_F64 ? 16 : 8) * (p->G_self[0] != 0.0 || p->G_self[1] != 0.0 ? 2 : 1);
+  return (int64_t)p->nx * p->ny * p->nz <= (int64_t(1) << 32) / site;
 }
-// ... and does: the step kernel is left to the library (no variant, tile or pipeline asked for), and either
-// the lattice cannot take the staged kernel, or it is FP64 (no density is summed twice), or the moments stay
-// in L2 between the passes.  Staged -> two passes, us a step: FP32 64^3 21.3 -> 11.9, 128^3 120.0 -> 117.6,
-// 160^3 227 -> 227, 256^3 884 -> 887; FP16 96^3 44.3 -> 37.8, 128^3 90.0 -> 91.8 (with a self coupling, whose
-// psi the one-pass kernel evaluates again in every halo, 107.5 -> 96.8, 160^3 185.4 -> 185.9).
+// ... and does: the step kernel is left to the library (no variant, tile or pipeline asked for), and the lattice
+// cannot take the staged kernel, or is FP64 (no density is summed twice), or is small enough.  Staged -> two passes,
+// us a step, without a self coupling: FP32 64^3 21.3 -> 11.9, 128^3 120.3 -> 107.8, 160^3 227.9 -> 220.5, 192^3 381.6 ->
+// 380.4, 320^3 1691 -> 1717; FP16 128^3 91.5 -> 84.5, 160^3 176.1 -> 168.9, 192^3 286.5 -> 289.5, 320^3 1243 -> 1313.
+// With one, whose psi the staged kernel evaluates again in every halo: FP32 320^3 1837 -> 1782, FP16 1499 -> 1404,
+// 512^3 5707 -> 5799.
 bool split_asked(const sc_params *p) {
   return split_eligible(p) && !p->variant && !p->tile_y && !p->tile_z && !p->stages && !p->blocks_per_sm;
 }
@@ -134,7 +136,7 @@ bool split_default(const sc_params *p) {
   if (!split_asked(p)) return false;
   if (!use_staged(p) || p->storage == SC_STORE_F64) return true;
   const int64_t sites = (int64_t)p->nx * p->ny * p->nz;
-  return sites <= (is_16bit(p->storage) && !has_self(p) ? int64_t(3) << 19 : int64_t(3) << 20);
+  return sites <= (has_self(p) ? int64_t(1) << 25 : int64_t(9) << 19);
 }
 
 sc_status validate(const sc_params *p) {

@@ -12,9 +12,9 @@
 // sides are (no lane idles in a partial x tile), and no block waits at a barrier; in return 32 bytes a site
 // (40 with a self coupling; twice that in FP64) are written and read again between the passes, through L2
 // while that buffer fits there.
-// Measured, one step, one-pass -> two passes (FP32 unless noted): E6 64 x 64 x 256 80.3 -> 68.2 us,
-// E6 160^3 302 -> 259 us (FP16 363 -> 209 us), 65^3 29.5 -> 15.1 us (paper couplings), 201^3 567 -> 497 us,
-// 64^3 21.4 -> 11.9 us, FP64 64^3 284 -> 191 us.  Bound: HBM at large sizes (256^3: 368 bytes a site at
+// Measured, one step, one-pass -> two passes (FP32 unless noted): E6 64 x 64 x 256 80.3 -> 58.0 us,
+// E6 160^3 302 -> 259 us (FP16 363 -> 209 us), 65^3 29.5 -> 14.9 us (paper couplings), 201^3 567 -> 499 us,
+// 64^3 21.4 -> 12.0 us, FP64 64^3 320 -> 212 us (one psi).  Bound: HBM at large sizes (256^3: 368 bytes a site at
 // 6.9 TB/s), FP64 arithmetic in FP64, latency below about 40^3.
 #pragma once
 
@@ -27,7 +27,9 @@ template <class CT>
 struct SplitArgs {
   StepArgs<CT> a;
   int keep_moments, pad;  // L2 eviction priorities, see L2Policy
-  P2<CT> *mom;  // [4 or 5][N]: density deviation, momentum sums x, y, z, with a self coupling psi deviation
+  // Pairs: density deviations [N], or with a self coupling density and psi deviations side by side [N][2] (a
+  // stencil neighbour is then one 16-byte load, not two of 8 and two addresses), then momentum sums x, y, z [N].
+  P2<CT> *mom;
   SiteDiv div;
 };
 
@@ -86,6 +88,26 @@ __device__ __forceinline__ T *at(T *base, unsigned bytes) {
   return reinterpret_cast<T *>(reinterpret_cast<uintptr_t>(base) + bytes);
 }
 
+// Density and psi deviations of a site.
+template <class CT>
+struct DensityPsi {
+  P2<CT> n, psi;
+};
+__device__ __forceinline__ DensityPsi<float> load_density_psi(const float2 *p) {
+  const float4 v = *reinterpret_cast<const float4 *>(p);
+  return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ DensityPsi<double> load_density_psi(const double2 *p) { return {p[0], p[1]}; }
+__device__ __forceinline__ void store_density_psi(float2 *p, float2 n, float2 psi, unsigned long long pol) {
+  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(n.x), "f"(n.y), "f"(psi.x),
+               "f"(psi.y), "l"(pol)
+               : "memory");
+}
+__device__ __forceinline__ void store_density_psi(double2 *p, double2 n, double2 psi, unsigned long long pol) {
+  store_hint(p, n, pol);
+  store_hint(p + 1, psi, pol);
+}
+
 // Moments pass at site s.
 template <class ST, class CT>
 __device__ __forceinline__ void split_moments(const SplitArgs<CT> &m, const ST *src, const float2 *nsrc, int s) {
@@ -119,12 +141,14 @@ __device__ __forceinline__ void split_moments(const SplitArgs<CT> &m, const ST *
   P2<CT> j[3];
   momentum_sums<kD3Q19, CT>(g, j);
   const unsigned p = unsigned(s) * unsigned(sizeof(P2<CT>));
-  store_hint(at(m.mom, p), dn, pol.last);
-  store_hint(at(m.mom + a.N, p), j[0], pol.last);
-  store_hint(at(m.mom + 2 * a.N, p), j[1], pol.last);
-  store_hint(at(m.mom + 3 * a.N, p), j[2], pol.last);
   if (a.self_on)
-    store_hint(at(m.mom + 4 * a.N, p), psi_deviation<CT>(dn, a.nbar, a.psibar, a.psi_exp, a.gself), pol.last);
+    store_density_psi(at(m.mom, 2 * p), dn, psi_deviation<CT>(dn, a.nbar, a.psibar, a.psi_exp, a.gself), pol.last);
+  else
+    store_hint(at(m.mom, p), dn, pol.last);
+  P2<CT> *jp = m.mom + (a.self_on ? 2 : 1) * a.N;
+  store_hint(at(jp, p), j[0], pol.last);
+  store_hint(at(jp + a.N, p), j[1], pol.last);
+  store_hint(at(jp + 2 * a.N, p), j[2], pol.last);
 }
 
 // Collision pass at site s: Eq. sc_force from the stored densities in force_pair's order, then the shared collision.
@@ -137,39 +161,52 @@ __device__ __forceinline__ void split_collide(const SplitArgs<CT> &m, ST *dst, f
   const L2Policy pol(m.keep_moments);
   int x, y, z;
   m.div.coords(s, a.nx, a.ny, x, y, z);
-  constexpr int E = sizeof(P2<CT>);
-  const unsigned o = unsigned(s) * E;
-  const P2<CT> *dnp = m.mom, *psp = m.mom + 4 * a.N;
-  const CT *jp = reinterpret_cast<const CT *>(m.mom);
-  const P2<CT> j[3] = {load_hint(at(jp + 2 * a.N, o), pol.first), load_hint(at(jp + 4 * a.N, o), pol.first),
-                       load_hint(at(jp + 6 * a.N, o), pol.first)};
-  const P2<CT> dn = *at(dnp, o);
-  const P2<CT> n = padd(a.nbar, dn);
-  unsigned X[2 * H + 1], Y[2 * H + 1], Z[2 * H + 1];  // byte offsets
+  constexpr unsigned E = sizeof(P2<CT>);
+  const unsigned p = unsigned(s) * E, E1 = a.self_on ? 2 * E : E, o = unsigned(s) * E1;  // byte offsets
+  const CT *jp = reinterpret_cast<const CT *>(m.mom + (a.self_on ? 2 : 1) * a.N);
+  const P2<CT> j[3] = {load_hint(at(jp, p), pol.first), load_hint(at(jp + 2 * a.N, p), pol.first),
+                       load_hint(at(jp + 4 * a.N, p), pol.first)};
+  unsigned X[2 * H + 1], Y[2 * H + 1], Z[2 * H + 1];
   const int W = a.nx * a.ny;
 #pragma unroll
   for (int d = -H; d <= H; ++d) {
-    X[d + H] = unsigned(wrapi(x + d, a.nx) - x) * E;
-    Y[d + H] = unsigned((wrapi(y + d, a.ny) - y) * a.nx) * E;
-    Z[d + H] = unsigned((wrapi(z + d, a.nz) - z) * W) * E;
+    X[d + H] = unsigned(wrapi(x + d, a.nx) - x) * E1;
+    Y[d + H] = unsigned((wrapi(y + d, a.ny) - y) * a.nx) * E1;
+    Z[d + H] = unsigned((wrapi(z + d, a.nz) - z) * W) * E1;
   }
+  const P2<CT> *mom = m.mom;
   P2<CT> S[3] = {pbc(CT(0)), pbc(CT(0)), pbc(CT(0))}, T[3] = {pbc(CT(0)), pbc(CT(0)), pbc(CT(0))};
+  P2<CT> dn, psi = pbc(CT(0));
+  if (a.self_on) {
+    const DensityPsi<CT> own = load_density_psi(at(mom, o));
+    dn = own.n;
+    psi = padd(a.psibar, own.psi);
 #pragma unroll
-  for (int k = 0; k < SN::NH; ++k) {
-    const int vx = SN::v(k, 0), vy = SN::v(k, 1), vz = SN::v(k, 2);
-    const unsigned ip = o + X[H + vx] + Y[H + vy] + Z[H + vz], im = o + X[H - vx] + Y[H - vy] + Z[H - vz];
-    const P2<CT> d = psub(*at(dnp, ip), *at(dnp, im));
-    if (vx) S[0] = pfma(pbc(CT(SN::W(k) * vx)), d, S[0]);
-    if (vy) S[1] = pfma(pbc(CT(SN::W(k) * vy)), d, S[1]);
-    if (vz) S[2] = pfma(pbc(CT(SN::W(k) * vz)), d, S[2]);
-    if (a.self_on) {
-      const P2<CT> e = psub(*at(psp, ip), *at(psp, im));
+    for (int k = 0; k < SN::NH; ++k) {
+      const int vx = SN::v(k, 0), vy = SN::v(k, 1), vz = SN::v(k, 2);
+      const DensityPsi<CT> fp = load_density_psi(at(mom, o + X[H + vx] + Y[H + vy] + Z[H + vz])),
+                           fm = load_density_psi(at(mom, o + X[H - vx] + Y[H - vy] + Z[H - vz]));
+      const P2<CT> d = psub(fp.n, fm.n), e = psub(fp.psi, fm.psi);
+      if (vx) S[0] = pfma(pbc(CT(SN::W(k) * vx)), d, S[0]);
+      if (vy) S[1] = pfma(pbc(CT(SN::W(k) * vy)), d, S[1]);
+      if (vz) S[2] = pfma(pbc(CT(SN::W(k) * vz)), d, S[2]);
       if (vx) T[0] = pfma(pbc(CT(SN::W(k) * vx)), e, T[0]);
       if (vy) T[1] = pfma(pbc(CT(SN::W(k) * vy)), e, T[1]);
       if (vz) T[2] = pfma(pbc(CT(SN::W(k) * vz)), e, T[2]);
     }
+  } else {
+    dn = *at(mom, o);
+#pragma unroll
+    for (int k = 0; k < SN::NH; ++k) {
+      const int vx = SN::v(k, 0), vy = SN::v(k, 1), vz = SN::v(k, 2);
+      const P2<CT> d = psub(*at(mom, o + X[H + vx] + Y[H + vy] + Z[H + vz]),
+                            *at(mom, o + X[H - vx] + Y[H - vy] + Z[H - vz]));
+      if (vx) S[0] = pfma(pbc(CT(SN::W(k) * vx)), d, S[0]);
+      if (vy) S[1] = pfma(pbc(CT(SN::W(k) * vy)), d, S[1]);
+      if (vz) S[2] = pfma(pbc(CT(SN::W(k) * vz)), d, S[2]);
+    }
   }
-  const P2<CT> psi = a.self_on ? padd(a.psibar, *at(psp, o)) : pbc(CT(0));
+  const P2<CT> n = padd(a.nbar, dn);
   const P2<CT> cn = pmul(pbc(a.gcross), n), cp = pmul(a.gself, psi);
   P2<CT> F[3], h[3], out[L::Q];
 #pragma unroll

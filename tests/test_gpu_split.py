@@ -55,7 +55,7 @@ def test_one_pass_kernels_keep_what_two_passes_cannot_take(B):
     kw = dict(G=2.5, psi_self=B.SC_PSI_EXP)
     for shape, extra, variant in (((3, 8, 8), {}, 1), ((8, 8, 3), {}, 1), ((16, 16, 16), dict(tau=(1.0, 0.9)), 1),
                                   ((16, 16, 1), dict(lattice=B.SC_D2Q9), 1), ((32, 32, 32), dict(tile_y=8), 2),
-                                  ((32, 32, 32), dict(variant=2), 2), ((160, 160, 160), {}, 2)):
+                                  ((32, 32, 32), dict(variant=2), 2), ((192, 192, 192), {}, 2)):
         sim = B.Simulation(B.make_params(shape, **kw, **extra), *field(shape, 7))
         assert sim.step_config["variant"] == variant, (shape, extra)
         sim.step(2)
