@@ -449,8 +449,8 @@ class _Member(Simulation):
 
 
 class Batch:
-    """Several lattices stepped together: one kernel launch per time step, or one
-    persistent launch per 32 steps for a staged batch."""
+    """Several lattices stepped together: in two passes per time step (the library's choice),
+    one launch per step, or one persistent launch per 32 steps for a staged batch."""
 
     def __init__(self, params_list, fields, device="cuda", stream=None):
         self.params = list(params_list)

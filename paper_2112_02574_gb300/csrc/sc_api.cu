@@ -124,17 +124,18 @@ bool split_eligible(const sc_params *p) {
   return (int64_t)p->nx * p->ny * p->nz <= (int64_t(1) << 32) / site;
 }
 // ... and does: the step kernel is left to the library (no variant, tile or pipeline asked for), and the lattice
-// cannot take the staged kernel, or is FP64 (no density is summed twice), or is small enough.  Staged -> two passes,
-// us a step, without a self coupling: FP32 64^3 21.3 -> 11.9, 128^3 120.3 -> 107.8, 160^3 227.9 -> 220.5, 192^3 381.6 ->
-// 380.4, 320^3 1691 -> 1717; FP16 128^3 91.5 -> 84.5, 160^3 176.1 -> 168.9, 192^3 286.5 -> 289.5, 320^3 1243 -> 1313.
-// With one, whose psi the staged kernel evaluates again in every halo: FP32 320^3 1837 -> 1782, FP16 1499 -> 1404,
-// 512^3 5707 -> 5799.
+// cannot take the staged kernel, or is FP64 or 16-bit, or is small enough in FP32.  Staged -> two passes, us a step,
+// without a self coupling: FP32 64^3 21.3 -> 11.9, 128^3 120.3 -> 107.8, 160^3 227.9 -> 220.5, 192^3 381.6 -> 380.4,
+// 320^3 1691 -> 1717; FP16 128^3 91.5 -> 80.4, 192^3 286.5 -> 275.9, 256^3 652 -> 636, 320^3 1243 -> 1240; BF16 256^3
+// 648 -> 637, 320^3 1237 -> 1242.  With one, whose psi the staged kernel evaluates again in every halo: FP32 320^3
+// 1837 -> 1782, 512^3 7207 -> 7313; FP16 320^3 1499 -> 1334, 512^3 5717 -> 5511; BF16 512^3 5689 -> 5547.
 bool split_asked(const sc_params *p) {
   return split_eligible(p) && !p->variant && !p->tile_y && !p->tile_z && !p->stages && !p->blocks_per_sm;
 }
 bool split_default(const sc_params *p) {
   if (!split_asked(p)) return false;
   if (!use_staged(p) || p->storage == SC_STORE_F64) return true;
+  if (is_16bit(p->storage)) return true;
   const int64_t sites = (int64_t)p->nx * p->ny * p->nz;
   return sites <= (has_self(p) ? int64_t(1) << 25 : int64_t(9) << 19);
 }

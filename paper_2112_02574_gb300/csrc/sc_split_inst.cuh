@@ -11,8 +11,10 @@ cudaError_t launch_split(int sten, const SplitArgs<CT> &m, cudaStream_t st) {
   const unsigned blocks = (unsigned)((m.a.N + kSplitThreads - 1) / kSplitThreads);
   cudaError_t e = launch_pass(sc_split_moments<ST, CT>, blocks, kSplitThreads, 0, st, m);
   if (e != cudaSuccess) return e;
-  return launch_pass(sten == kE6 ? sc_split_collide<kE6, ST, CT> : sc_split_collide<kE4, ST, CT>, blocks,
-                     kSplitThreads, 0, st, m);
+  const bool small = sizeof(CT) == 4 && m.a.self_on && m.a.N <= kSmallCollide;
+  auto *collide = sten == kE6 ? (small ? sc_split_collide<kE6, ST, CT, true> : sc_split_collide<kE6, ST, CT, false>)
+                              : (small ? sc_split_collide<kE4, ST, CT, true> : sc_split_collide<kE4, ST, CT, false>);
+  return launch_pass(collide, blocks, kSplitThreads, 0, st, m);
 }
 
 template <class ST, class CT>

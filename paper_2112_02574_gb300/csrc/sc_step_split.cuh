@@ -222,23 +222,29 @@ __device__ __forceinline__ void split_collide(const SplitArgs<CT> &m, ST *dst, f
   if constexpr (local_ref<ST>()) *at(ndst, unsigned(s) * 8u) = make_float2(float(dn.x), float(dn.y));
 }
 
-// Threads per block and the blocks per SM the register allocation must allow (64 registers a thread, 80 for
-// the 33 neighbours of E6 in a batch, which would spill; 128 in FP64).  128 threads against 256: 1-2 %
-// faster from 64^3 up, equal below.
+// Threads per block and the blocks per SM the register allocation must allow: eight (64 registers a thread), in FP64
+// four (128).  128 threads against 256: 1-2 % faster from 64^3 up, equal below.  Six blocks (80 registers, more loads
+// in flight per thread) for
+//  * the FP16 moments, whose 19 pairs and 19 references a thread wait for each other otherwise: 128^3 84.5 -> 80.0 us
+//    a step, with psi 95.2 -> 90.2, 256^3 with psi 724 -> 688 (BF16 and FP32: no change);
+//  * the collisions of a small lattice with psi (16 bytes a neighbour), whose few waves are bound by latency: 51^3
+//    10.1 -> 9.0, 65^3 15.0 -> 14.5; larger ones lose 2 % (128^3 115.1 -> 117.3);
+//  * the 33 neighbours of E6 in a batch, which would spill.
 constexpr int kSplitThreads = 128;
+constexpr int kSmallCollide = 300000;  // sites
 template <class CT>
-constexpr int split_blocks(bool spills = false) { return sizeof(CT) == 8 ? 4 : (spills ? 6 : 8); }
+constexpr int split_blocks(bool six = false) { return sizeof(CT) == 8 ? 4 : (six ? 6 : 8); }
 
 template <class ST, class CT>
-__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>())
+__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>(std::is_same<ST, __half>::value))
     sc_split_moments(const __grid_constant__ SplitArgs<CT> m) {
   const int s = blockIdx.x * kSplitThreads + threadIdx.x;
   pass_begin();
   if (s < m.a.N) split_moments<ST, CT>(m, static_cast<const ST *>(m.a.src), m.a.nsrc, s);
 }
 
-template <int STEN, class ST, class CT>
-__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>())
+template <int STEN, class ST, class CT, bool SMALL>
+__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>(SMALL))
     sc_split_collide(const __grid_constant__ SplitArgs<CT> m) {
   const int s = blockIdx.x * kSplitThreads + threadIdx.x;
   pass_begin();
@@ -260,7 +266,7 @@ __device__ __forceinline__ void split_fetch(SplitArgs<CT> &m, const SplitArgs<CT
 }
 
 template <class ST, class CT>
-__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>())
+__global__ void __launch_bounds__(kSplitThreads, split_blocks<CT>(std::is_same<ST, __half>::value))
     sc_split_moments_batched(const SplitArgs<CT> *args, const int2 *items, int swap) {
   __shared__ SplitArgs<CT> m;
   const int2 it = items[blockIdx.x];

@@ -1,8 +1,7 @@
 """Tolman length and rigidity from a sweep of droplets (section 4, Eq. sigma_c).
 
 Droplets of several radii, rich in component A (positive curvature) or in B
-(negative curvature), are stepped together as one batch (one step-kernel launch
-per time step).  For each member the device computes the radial pressure-tensor
+(negative curvature), are stepped together as one batch.  For each member the device computes the radial pressure-tensor
 profile (Eq. sm:pt), the bulk pressures at the centre node and at the far corner
 (Eq. bulkp) and the sigma[R] minimum (Eqs. gen_sigma, gen_d_sigma), which give
 (R_s, sigma_s = dP R_s / 2).  A periodic slab gives the flat-interface tension
