@@ -38,7 +38,8 @@ LOCAL_REF_BYTES = {"f16": 16, "bf16": 16}
 # DRAM bytes (read + write) of one step launch on this workload, from an ncu capture of the
 # launch; reported only while the kernel sources still hash to the captured version.
 KERNEL_SOURCES = ["paper_2112_02574_gb300/csrc/sc_common.cuh", "paper_2112_02574_gb300/csrc/sc_step_kernel.cuh",
-                  "paper_2112_02574_gb300/csrc/sc_step_staged.cuh"]
+                  "paper_2112_02574_gb300/csrc/sc_step_staged.cuh", "paper_2112_02574_gb300/csrc/sc_step_split.cuh"]
+STEP_KERNELS = {1: "sc_step_kernel", 2: "sc_step_staged", 3: "sc_split_moments + sc_split_collide"}
 # DRAM bytes per step launch (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture), keyed by the
 # kernel sources' hash, the storage and the launch (tile_y, stages, blocks_per_sm, blocks); a change to any of
 # them drops the figure (reported as null) until it is measured again
@@ -318,8 +319,9 @@ def run_gpu(args, rank, world, local_rank):
     if dist:
         ms = max_over_ranks(ms, dev)
     step_launches = sim.launches - launches0
-    # per bench step: INNER fused steps + fields + profile partials + profile finalise + 2 bulk + sigma
-    launches = step_launches + args.steps * 6
+    # per bench step: INNER time steps (one launch each, two with the two-pass step) + fields + profile partials +
+    # profile finalise + 2 bulk + sigma
+    launches = step_launches * (2 if step_cfg["variant"] == 3 else 1) + args.steps * 6
 
     # kernel-only timing of the fused step (events around the INNER launches, separate pass)
     if not step_ms:
@@ -383,7 +385,7 @@ def run_gpu(args, rank, world, local_rank):
         "vs_baseline": None, "dtype": storage, "data": "synthetic", "config": workload_config(storage),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "traffic": MEASURED_TRAFFIC.get((kernel_hash(), storage, traffic_key(step_cfg))),
-                     "kernel": "sc_step_staged" if step_cfg["variant"] == 2 else "sc_step_kernel",
+                     "kernel": STEP_KERNELS[step_cfg["variant"]],
                      "launch": step_cfg,
                      "bytes_per_site": BYTES_PER_SITE[storage], "algorithmic_bytes_per_launch": alg_bytes,
                      "kernel_ms": kern_ms, "peak_source": peak_kind,
@@ -418,7 +420,8 @@ def sweep_droplets():
     return out
 
 
-BATCH_CANDIDATES = [(8, 64, 1, 3), (8, 32, 1, 3), (8, 64, 1, 2), (4, 32, 1, 3), (4, 64, 1, 3), (4, 128, 1, 3),
+# the first leaves the step kernel to the library (two passes)
+BATCH_CANDIDATES = [(0, 0, 0, 0), (8, 64, 1, 3), (8, 32, 1, 3), (8, 64, 1, 2), (4, 32, 1, 3), (4, 64, 1, 3), (4, 128, 1, 3),
                     (4, 64, 2, 2)]
 
 
