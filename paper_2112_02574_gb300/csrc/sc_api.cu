@@ -669,7 +669,7 @@ sc_status sc_create(const sc_params *params, const double *nA0, const double *nB
   c->split = split_default(params) ? 1 : 0;
   c->lanes = use_lanes(params) ? 1 : 0;
   if (c->lanes) c->tile_y = 1;
-  if (params->tile_z == 0 && params->lattice == SC_D3Q19) {
+  if (!c->split && params->tile_z == 0 && params->lattice == SC_D3Q19) {
     st = plan_z_split(c);
     if (st != SC_OK) {
       delete c;
