@@ -563,6 +563,7 @@ sc_status launch_one_step(sc_ctx *c) {
   l.stream = c->stream;
   cudaError_t e;
   if (c->split) {
+    c->fields_at = -1;  // the moments take the fields' space, also where the collision then fails to launch
     e = launch_split_step(c, c->cur, c->stream);
   } else if (c->lanes) {
     e = launch_step_lanes(step_args<double>(c), c->stream);
@@ -574,7 +575,10 @@ sc_status launch_one_step(sc_ctx *c) {
       default: e = launch_step_f64(l, step_args<double>(c)); break;
     }
   }
-  if (e != cudaSuccess) return fail(SC_ECUDA, "step kernel launch: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next call
+    return fail(SC_ECUDA, "step kernel launch: %s", cudaGetErrorString(e));
+  }
   c->cur = 1 - c->cur;
   c->launches++;
   c->steps++;
@@ -1560,6 +1564,9 @@ sc_status sc_batch_step(sc_batch *b, int64_t nsteps) {
   if (!b) return fail(SC_EINVAL, "batch is NULL");
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
   if (b->nitems == 0) return SC_OK;  // every member retired
+  if (b->split && nsteps > 0)  // the moments take the fields' space, also in a step that fails half way
+    for (int k = 0; k < b->n; ++k)
+      if (!b->retired[k]) b->ctx[k]->fields_at = -1;
   auto single = [&]() -> cudaError_t {
     if (b->split) {
       cudaError_t e = cudaSuccess;
