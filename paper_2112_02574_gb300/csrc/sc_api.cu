@@ -1567,42 +1567,40 @@ sc_status sc_batch_step(sc_batch *b, int64_t nsteps) {
   if (b->split && nsteps > 0)  // the moments take the fields' space, also in a step that fails half way
     for (int k = 0; k < b->n; ++k)
       if (!b->retired[k]) b->ctx[k]->fields_at = -1;
+  // A step reads one buffer of every member and writes the other, so one that fails to launch (between two groups
+  // as well) leaves the state before it: it is not counted, and the next call runs it again.
   auto single = [&]() -> cudaError_t {
+    const int swap = (int)(b->steps & 1);
     if (b->split) {
       cudaError_t e = cudaSuccess;
-      for (int g = 0; g < b->ngroups && e == cudaSuccess; ++g)
-        e = batch_split_step(b, g, (int)(b->steps & 1), b->stream);
-      b->steps++;
-      b->launches++;
+      for (int g = 0; g < b->ngroups && e == cudaSuccess; ++g) e = batch_split_step(b, g, swap, b->stream);
       return e;
     }
     void *argp = b->args_dev;
     void *itemp = b->items_dev;
-    int swap = (int)(b->steps & 1);
-    void *kp[3] = {&argp, &itemp, &swap};
-    cudaError_t e = cudaLaunchKernel(b->kernel, dim3(b->nitems), dim3(32, b->tile_y), kp, b->smem, b->stream);
-    b->steps++;
-    b->launches++;
-    return e;
+    int swaparg = swap;
+    void *kp[3] = {&argp, &itemp, &swaparg};
+    return cudaLaunchKernel(b->kernel, dim3(b->nitems), dim3(32, b->tile_y), kp, b->smem, b->stream);
   };
+  cudaError_t e = cudaSuccess;
   while (nsteps > 0) {
-    cudaError_t e;
-    if ((b->steps & 1) == 0 && nsteps >= kGraphSteps) {
-      e = cudaGraphLaunch(b->exec, b->stream);
-      b->steps += kGraphSteps;
-      b->launches += kGraphSteps;
-      nsteps -= kGraphSteps;
-    } else {
-      e = single();
-      nsteps -= 1;
-    }
-    if (e != cudaSuccess) return fail(SC_ECUDA, "batched step: %s", cudaGetErrorString(e));
+    const bool run = (b->steps & 1) == 0 && nsteps >= kGraphSteps;
+    e = run ? cudaGraphLaunch(b->exec, b->stream) : single();
+    if (e != cudaSuccess) break;
+    const int64_t done = run ? kGraphSteps : 1;
+    b->steps += done;
+    b->launches += done;
+    nsteps -= done;
   }
   for (int k = 0; k < b->n; ++k) {
     if (b->retired[k]) continue;
     b->ctx[k]->cur = (int)(b->steps & 1);
     b->ctx[k]->steps = b->steps;
     b->ctx[k]->launches = b->launches;
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next call
+    return fail(SC_ECUDA, "batched step: %s", cudaGetErrorString(e));
   }
   return SC_OK;
 }

@@ -45,3 +45,34 @@ def test_two_pass_step_that_fails_half_way_leaves_no_fields_behind(B, L):
     assert ["moments" in n for n in fake_gpu.calls(L)] == [True]
     assert L.sc_kernel_launches(c.ctx) == 0
     assert c.moments() == B.SC_OK and fields_computed(L) == 1
+
+
+def test_batch_step_that_fails_is_not_counted(B, L):
+    """A step that fails between the groups of a two-pass batch is not counted, and run again from the same buffers (a
+    step reads one buffer and writes the other); no member's fields are taken from before it."""
+    b = fake_gpu.Batch(L, [B.make_params((96, 96, 96), G=2.5), B.make_params((16, 16, 16), G=2.5)])
+    assert b.status == B.SC_OK and L.sc_batch_variant(b.handle) == 4
+    m = [b.member(k) for k in range(2)]
+    keep, out = fake_gpu.buffer(16 * 96**3)
+    for x in m:
+        assert L.sc_moments(x, out, out, None) == B.SC_OK
+    L.fake_reset()
+    L.fake_fail(b"kernel", 5)  # one step (two groups of two launches), then the second's first group only
+    assert L.sc_batch_step(b.handle, 3) == B.SC_ECUDA
+    assert L.sc_batch_launches(b.handle) == 1
+    assert [L.sc_kernel_launches(x) for x in m] == [1, 1]
+    before = fields_computed(L)
+    for x in m:
+        assert L.sc_moments(x, out, out, None) == B.SC_OK
+    assert fields_computed(L) == before + 2
+    assert L.sc_batch_step(b.handle, 2) == B.SC_OK
+    assert L.sc_batch_launches(b.handle) == 3
+    assert [L.sc_kernel_launches(x) for x in m] == [3, 3]
+
+
+def test_batch_run_that_fails_is_not_counted(B, L):
+    b = fake_gpu.Batch(L, [B.make_params((16, 16, 16), G=2.5)])
+    L.fake_fail(b"cudaGraphLaunch", 1)
+    assert L.sc_batch_step(b.handle, 96) == B.SC_ECUDA
+    assert L.sc_batch_launches(b.handle) == 32
+    assert L.sc_kernel_launches(b.member(0)) == 32
