@@ -1372,8 +1372,13 @@ sc_status batch_build_graph(sc_batch *b) {
   b->pgrid = 0;
   if (b->nitems == 0) return SC_OK;
   if (b->split) {
-    const cudaError_t e = batch_capture_split(b);
-    if (e != cudaSuccess) return fail(SC_ECUDA, "building the batch graph: %s", cudaGetErrorString(e));
+    if (batch_capture_split(b) != cudaSuccess) {  // no graph: every step is plain launches
+      if (b->exec) cudaGraphExecDestroy(b->exec);
+      if (b->graph) cudaGraphDestroy(b->graph);
+      b->exec = nullptr;
+      b->graph = nullptr;
+      cudaGetLastError();  // the capture's error is not the caller's
+    }
     return SC_OK;
   }
   if (b->pkernel && !b->persist_off && batch_build_persistent(b)) return SC_OK;
@@ -1584,7 +1589,7 @@ sc_status sc_batch_step(sc_batch *b, int64_t nsteps) {
   };
   cudaError_t e = cudaSuccess;
   while (nsteps > 0) {
-    const bool run = (b->steps & 1) == 0 && nsteps >= kGraphSteps;
+    const bool run = b->exec && (b->steps & 1) == 0 && nsteps >= kGraphSteps;
     e = run ? cudaGraphLaunch(b->exec, b->stream) : single();
     if (e != cudaSuccess) break;
     const int64_t done = run ? kGraphSteps : 1;

@@ -76,3 +76,28 @@ def test_batch_run_that_fails_is_not_counted(B, L):
     assert L.sc_batch_step(b.handle, 96) == B.SC_ECUDA
     assert L.sc_batch_launches(b.handle) == 32
     assert L.sc_kernel_launches(b.member(0)) == 32
+
+
+def test_two_pass_batch_without_a_graph_steps_with_plain_launches(B, L):
+    """Where the capture of a run fails, creating the batch and retiring a member succeed and whole runs go out as
+    plain launches (two per group and step), as a lone context's do."""
+    params = [B.make_params((16, 16, 16), G=2.5), B.make_params((96, 96, 96), G=2.5)]
+    for call in (b"cudaStreamCreateWithFlags", b"cudaStreamBeginCapture", b"kernel", b"cudaGraphInstantiate"):
+        L.fake_reset()
+        whole = fake_gpu.Batch(L, params)
+        assert whole.status == B.SC_OK
+        L.fake_fail(call, 0)
+        assert L.sc_batch_retire(whole.handle, 0) == B.SC_OK
+        L.fake_reset()
+        assert L.sc_batch_step(whole.handle, 34) == B.SC_OK
+        assert len(fake_gpu.calls(L)) == 2 * 34 and "graph launch" not in fake_gpu.calls(L)
+        assert L.sc_batch_launches(whole.handle) == 34
+        L.sc_batch_destroy(whole.handle)
+    for call in (b"cudaStreamCreateWithFlags", b"cudaGraphInstantiate"):
+        L.fake_reset()
+        L.fake_fail(call, 0)
+        b = fake_gpu.Batch(L, params)
+        assert b.status == B.SC_OK and L.sc_batch_variant(b.handle) == 4
+        L.fake_reset()
+        assert L.sc_batch_step(b.handle, 32) == B.SC_OK
+        assert len(fake_gpu.calls(L)) == 4 * 32
