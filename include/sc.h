@@ -336,10 +336,14 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
 /* Advance every member by nsteps time steps (section 2); asynchronous. */
 sc_status sc_batch_step(sc_batch *batch, int64_t nsteps);
 /* Choose how whole runs of 32 steps of a staged batch go out: on = 1 (the
- * default where the device has cooperative launch) one persistent launch per
- * run, on = 0 one launch per step.  Both forms give the same members bit for
- * bit.  Waits for the batch's stream.  SC_EUNSUPPORTED for on = 1 when the
- * batch has no persistent form (a generic batch, or no cooperative launch). */
+ * default of a staged batch that does not step in two passes, where the device
+ * has cooperative launch) one persistent launch per run, on = 0 one launch per
+ * step.  A batch that steps in two passes ignores on = 0, having no persistent
+ * launch; on = 1 makes it a staged batch for good (a later on = 0 then means one
+ * launch per step).  Every form gives the same members bit for bit.  Waits for
+ * the batch's stream.  SC_EUNSUPPORTED for on = 1 when the batch has no
+ * persistent form (a generic batch, or no cooperative launch) or it cannot be
+ * built; the batch then steps as before the call. */
 sc_status sc_batch_set_persistent(sc_batch *batch, int32_t on);
 /* Member k as a context (owned by the batch; NULL if k is out of range). */
 sc_ctx *sc_batch_member(sc_batch *batch, int32_t k);

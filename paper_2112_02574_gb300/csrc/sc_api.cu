@@ -1630,11 +1630,18 @@ sc_status sc_batch_set_persistent(sc_batch *b, int32_t on) {
   if (on && !b->pkernel) return fail(SC_EUNSUPPORTED, "the batch has no persistent form (generic kernel or no cooperative launch)");
   if (b->split && !on) return SC_OK;  // no persistent launch in use
   SC_CUDA(cudaStreamSynchronize(b->stream));
+  const int split = b->split;
   b->persist_off = !on;
   b->split = 0;
   sc_status st = batch_build_graph(b);
   if (st == SC_OK && on && b->nitems > 0 && b->pgrid == 0)
-    return fail(SC_EUNSUPPORTED, "the persistent launch could not be built on this device");
+    st = fail(SC_EUNSUPPORTED, "the persistent launch could not be built on this device");
+  if (st != SC_OK && split) {  // the two passes stay
+    const std::string why = g_err;
+    b->split = split;
+    batch_build_graph(b);
+    g_err = why;
+  }
   return st;
 }
 

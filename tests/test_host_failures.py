@@ -101,3 +101,19 @@ def test_two_pass_batch_without_a_graph_steps_with_plain_launches(B, L):
         L.fake_reset()
         assert L.sc_batch_step(b.handle, 32) == B.SC_OK
         assert len(fake_gpu.calls(L)) == 4 * 32
+
+
+def test_failed_persistent_build_keeps_the_two_passes(B, L):
+    """SC_EUNSUPPORTED leaves the batch as it was; the form changes when the persistent launch has been built."""
+    b = fake_gpu.Batch(L, [B.make_params((32, 32, 32), G=2.5), B.make_params((40, 16, 12), G=2.5)])
+    assert b.status == B.SC_OK and L.sc_batch_variant(b.handle) == 4
+    L.fake_fail(b"cudaGraphInstantiate", 0)
+    assert L.sc_batch_set_persistent(b.handle, 1) == B.SC_EUNSUPPORTED
+    assert b"persistent" in L.sc_last_error()
+    assert L.sc_batch_variant(b.handle) == 4
+    L.fake_reset()
+    assert L.sc_batch_step(b.handle, 33) == B.SC_OK
+    assert [("split" in c) for c in fake_gpu.calls(L)] == [False, True, True]  # a replayed run, then one step
+    assert L.sc_batch_set_persistent(b.handle, 1) == B.SC_OK and L.sc_batch_variant(b.handle) == 3
+    # from here on the batch is a staged one: without the persistent launch it takes one launch per step
+    assert L.sc_batch_set_persistent(b.handle, 0) == B.SC_OK and L.sc_batch_variant(b.handle) == 2
