@@ -291,6 +291,7 @@ struct sc_ctx {
   int64_t launches;
   int64_t steps;
   int64_t fields_at;  // step count the FP64 fields were computed at (-1: stale)
+  int captured;       // a step went into a caller's graph, whose replays the step count does not see
   int in_batch;       // stepped by a batch (sc_step refuses)
   // kGraphSteps consecutive step launches from buffer 0, captured once on a private
   // stream and replayed on the context's stream (graph_failed: capture not possible,
@@ -399,9 +400,18 @@ int grid_for(int64_t n, int block) {
     }                                                                                                     \
   } while (0)
 
-// FP64 density / pseudopotential fields of the current state (cached per step count).
+// The stream records a caller's graph.  (False where the runtime cannot tell: the legacy stream beside a capture.)
+bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+
+// FP64 density / pseudopotential fields of the current state (cached per step count, except where the caller's
+// graphs may have stepped it).
 sc_status ensure_fields(sc_ctx *c) {
-  if (c->fields_at == c->steps) return SC_OK;
+  if (c->fields_at == c->steps && !c->captured) return SC_OK;
   PopArgs a = pop_args(c, c->cur);
   SC_POP_DISPATCH(c, fields_kernel, grid_for(c->N, 128), 128, 0, a, c->p.psi_self,
                   (c->p.G_self[0] != 0.0 ? 1 : 0) | (c->p.G_self[1] != 0.0 ? 2 : 0), fields_of(c));
@@ -765,6 +775,7 @@ sc_status sc_step(sc_ctx *c, int64_t nsteps) {
   if (!c) return fail(SC_EINVAL, "ctx is NULL");
   if (c->in_batch) return fail(SC_EINVAL, "this context belongs to a batch: step it with sc_batch_step");
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
+  if (nsteps > 0 && !c->captured) c->captured = is_capturing(c->stream) ? 1 : 0;
   while (nsteps > 0) {
     // runs of kStepGraphSteps from buffer 0 replay the step graph (built on first use,
     // once the kernel has launched normally)
@@ -1569,9 +1580,12 @@ sc_status sc_batch_step(sc_batch *b, int64_t nsteps) {
   if (!b) return fail(SC_EINVAL, "batch is NULL");
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
   if (b->nitems == 0) return SC_OK;  // every member retired
-  if (b->split && nsteps > 0)  // the moments take the fields' space, also in a step that fails half way
-    for (int k = 0; k < b->n; ++k)
-      if (!b->retired[k]) b->ctx[k]->fields_at = -1;
+  const bool captured = nsteps > 0 && is_capturing(b->stream);
+  for (int k = 0; k < b->n; ++k) {
+    if (b->retired[k] || nsteps == 0) continue;
+    if (b->split) b->ctx[k]->fields_at = -1;  // the moments take the fields' space, also in a step that fails half way
+    if (captured) b->ctx[k]->captured = 1;
+  }
   // A step reads one buffer of every member and writes the other, so one that fails to launch (between two groups
   // as well) leaves the state before it: it is not counted, and the next call runs it again.
   auto single = [&]() -> cudaError_t {

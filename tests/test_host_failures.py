@@ -117,3 +117,23 @@ def test_failed_persistent_build_keeps_the_two_passes(B, L):
     assert L.sc_batch_set_persistent(b.handle, 1) == B.SC_OK and L.sc_batch_variant(b.handle) == 3
     # from here on the batch is a staged one: without the persistent launch it takes one launch per step
     assert L.sc_batch_set_persistent(b.handle, 0) == B.SC_OK and L.sc_batch_variant(b.handle) == 2
+
+
+def test_fields_after_a_captured_step_are_computed_anew(B, L):
+    """A step recorded into a caller's graph runs again at every replay, which the library does not see: the fields it
+    leaves (the moments are in their space) are never taken for the cached ones."""
+    c = fake_gpu.Context(L, B.make_params((16, 16, 16), G=2.5))
+    L.fake_capturing(1)
+    assert L.sc_step(c.ctx, 2) == B.SC_OK
+    L.fake_capturing(0)
+    for k in range(3):  # with a replay before each
+        L.fake_reset()
+        assert c.moments() == B.SC_OK and fields_computed(L) == 1, k
+    b = fake_gpu.Batch(L, [B.make_params((16, 16, 16), G=2.5)])
+    out = fake_gpu.buffer(32 * 16**3)
+    L.fake_capturing(1)
+    assert L.sc_batch_step(b.handle, 2) == B.SC_OK
+    L.fake_capturing(0)
+    for k in range(2):
+        L.fake_reset()
+        assert L.sc_moments(b.member(0), out[1], out[1], None) == B.SC_OK and fields_computed(L) == 1, k
