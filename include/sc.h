@@ -104,7 +104,12 @@ typedef struct sc_ctx sc_ctx;
 
 /* Bytes of device workspace sc_create needs for these parameters (0 if the
  * parameters are invalid).  Layout: two population buffers, FP64 field planes
- * for the analysis kernels, reduction scratch and a status word. */
+ * for the analysis kernels, reduction scratch and a status word.  The two-pass
+ * step keeps its moments in the space of the field planes; where the library
+ * takes it (variant 0) they need 8 bytes a site more with a self coupling, in
+ * FP64 storage 32 (48 with a self coupling).  A workspace without that room (the
+ * bytes of the same parameters with variant = 1) serves too: the context, or
+ * the batch, then steps with the one-pass kernels. */
 size_t sc_workspace_bytes(const sc_params *params);
 
 /* Create a simulation (section 2; initial state of section 4: rest equilibrium

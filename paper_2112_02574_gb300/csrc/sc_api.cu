@@ -175,7 +175,8 @@ struct Layout {
 
 bool is_local_ref(int storage) { return storage == SC_STORE_F16 || storage == SC_STORE_BF16; }
 
-Layout layout_of(const sc_params *p) {
+// moments: with room for the moments of the two-pass step.
+Layout layout_of(const sc_params *p, bool moments) {
   Layout L;
   const int64_t N = (int64_t)p->nx * p->ny * p->nz;
   L.pop_bytes = (size_t)2 * q_of(p) * N * store_bytes(p->storage);
@@ -193,7 +194,7 @@ Layout layout_of(const sc_params *p) {
   // the FP64 fields and the moments of the two-pass step share this space: each is computed anew from the
   // populations before it is read
   size_t shared = (size_t)4 * N * sizeof(double);
-  if (split_eligible(p))
+  if (moments)
     shared = std::max(shared, (size_t)N * (p->storage == SC_STORE_F64 ? 16 : 8) * (has_self(p) ? 5 : 4));
   off = align_up(off + shared);
   L.off_partial = off;
@@ -651,18 +652,20 @@ extern "C" {
 
 size_t sc_workspace_bytes(const sc_params *params) {
   if (validate(params) != SC_OK) return 0;
-  return layout_of(params).total;
+  return layout_of(params, split_default(params)).total;
 }
 
-sc_status sc_create(const sc_params *params, const double *nA0, const double *nB0, void *workspace, size_t ws_bytes,
-                    void *stream, sc_ctx **out) {
-  if (!out) return fail(SC_EINVAL, "out is NULL");
+namespace {
+// A context; two_pass: its step takes two passes (or may, in a batch) if the workspace has room for their moments.
+sc_status create_context(const sc_params *params, const double *nA0, const double *nB0, void *workspace,
+                         size_t ws_bytes, void *stream, bool two_pass, sc_ctx **out) {
   *out = nullptr;
-  sc_status st = validate(params);
-  if (st != SC_OK) return st;
-  if (!nA0 || !nB0 || !workspace) return fail(SC_EINVAL, "initial fields and workspace must be non-NULL");
-  if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return fail(SC_EINVAL, "workspace must be 256-byte aligned");
-  Layout L = layout_of(params);
+  sc_status st;
+  Layout L = layout_of(params, two_pass);
+  if (ws_bytes < L.total && two_pass) {  // a workspace that serves the one-pass kernels still does
+    two_pass = layout_of(params, false).total == L.total;
+    if (!two_pass) L = layout_of(params, false);
+  }
   if (ws_bytes < L.total) return fail(SC_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, L.total);
   sc_ctx *c = new (std::nothrow) sc_ctx;
   if (!c) return fail(SC_ENOMEM, "host allocation failed");
@@ -680,7 +683,7 @@ sc_status sc_create(const sc_params *params, const double *nA0, const double *nB
   c->stages = effective_stages(params, c->tile_y);
   c->blocks_per_sm = effective_blocks_per_sm(params, c->tile_y);
   c->fields_at = -1;
-  c->split = split_default(params) ? 1 : 0;
+  c->split = two_pass && split_default(params) ? 1 : 0;
   c->lanes = use_lanes(params) ? 1 : 0;
   if (c->lanes) c->tile_y = 1;
   if (!c->split && params->tile_z == 0 && params->lattice == SC_D3Q19) {
@@ -728,6 +731,18 @@ sc_status sc_create(const sc_params *params, const double *nA0, const double *nB
   }
   *out = c;
   return SC_OK;
+}
+}  // namespace
+
+sc_status sc_create(const sc_params *params, const double *nA0, const double *nB0, void *workspace, size_t ws_bytes,
+                    void *stream, sc_ctx **out) {
+  if (!out) return fail(SC_EINVAL, "out is NULL");
+  *out = nullptr;
+  sc_status st = validate(params);
+  if (st != SC_OK) return st;
+  if (!nA0 || !nB0 || !workspace) return fail(SC_EINVAL, "initial fields and workspace must be non-NULL");
+  if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return fail(SC_EINVAL, "workspace must be 256-byte aligned");
+  return create_context(params, nA0, nB0, workspace, ws_bytes, stream, split_default(params), out);
 }
 
 namespace {
@@ -1067,7 +1082,7 @@ sc_status sc_run_host(const sc_params *params, const double *nA0, const double *
   if (st != SC_OK) return st;
   if (!nA0 || !nB0 || !nA || !nB || !workspace) return fail(SC_EINVAL, "buffers must be non-NULL");
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
-  Layout L = layout_of(params);
+  const Layout L = layout_of(params, false);
   if (ws_bytes < L.total) return fail(SC_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, L.total);
   const int64_t N = (int64_t)params->nx * params->ny * params->nz;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -1097,7 +1112,7 @@ sc_status sc_run_host_sigma(const sc_params *params, const double *nA0, const do
   if (st != SC_OK) return st;
   if (!nA0 || !nB0 || !result || !workspace) return fail(SC_EINVAL, "nA0, nB0, result and workspace must be non-NULL");
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
-  Layout L = layout_of(params);
+  const Layout L = layout_of(params, false);
   if (ws_bytes < L.total) return fail(SC_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, L.total);
   const int64_t N = (int64_t)params->nx * params->ny * params->nz;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -1179,7 +1194,7 @@ size_t split_table_bytes(int32_t n, const sc_params *params, int64_t *items_out)
   return align_up(sizeof(SplitArgs<double>) * (size_t)n) + align_up(sizeof(int2) * (size_t)items);
 }
 
-size_t batch_table_bytes(int32_t n, const sc_params *params, int *nitems_out) {
+size_t batch_table_bytes(int32_t n, const sc_params *params, bool split, int *nitems_out) {
   const bool staged = batch_staged(n, params);
   int nitems = 0;
   for (int k = 0; k < n; ++k) {
@@ -1189,7 +1204,14 @@ size_t batch_table_bytes(int32_t n, const sc_params *params, int *nitems_out) {
   }
   if (nitems_out) *nitems_out = nitems;
   return align_up(sizeof(StepArgs<double>) * (size_t)n) + align_up(sizeof(int4) * (size_t)nitems) + kAlign +
-         (batch_split(n, params) ? split_table_bytes(n, params, nullptr) : 0);
+         (split ? split_table_bytes(n, params, nullptr) : 0);
+}
+
+// Workspace of a batch that steps in two passes, or does not.
+size_t batch_bytes(int32_t n, const sc_params *params, bool split) {
+  size_t total = batch_table_bytes(n, params, split, nullptr);
+  for (int k = 0; k < n; ++k) total += layout_of(&params[k], split).total;
+  return total;
 }
 
 sc_status batch_validate(int32_t n, const sc_params *params) {
@@ -1419,9 +1441,7 @@ sc_status batch_build_graph(sc_batch *b) {
 
 size_t sc_batch_workspace_bytes(int32_t n, const sc_params *params) {
   if (batch_validate(n, params) != SC_OK) return 0;
-  size_t total = 0;
-  for (int k = 0; k < n; ++k) total += layout_of(&params[k]).total;
-  return total + batch_table_bytes(n, params, nullptr);
+  return batch_bytes(n, params, batch_split(n, params));
 }
 
 sc_status sc_batch_create(int32_t n, const sc_params *params, const double *const *nA0, const double *const *nB0,
@@ -1432,7 +1452,9 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
   if (st != SC_OK) return st;
   if (!nA0 || !nB0 || !workspace) return fail(SC_EINVAL, "initial fields and workspace must be non-NULL");
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return fail(SC_EINVAL, "workspace must be 256-byte aligned");
-  const size_t need = sc_batch_workspace_bytes(n, params);
+  bool split = batch_split(n, params);
+  if (split && ws_bytes < batch_bytes(n, params, true)) split = false;  // no room: the one-pass kernels
+  const size_t need = batch_bytes(n, params, split);
   if (ws_bytes < need) return fail(SC_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, need);
   sc_batch *b = new (std::nothrow) sc_batch;
   if (!b) return fail(SC_ENOMEM, "host allocation failed");
@@ -1450,8 +1472,10 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
   const bool staged = batch_staged(n, params);
   for (int k = 0; k < n; ++k) {
     sc_params pk = member_params(n, params, k, staged);
-    const size_t bytes = layout_of(&pk).total;
-    st = sc_create(&pk, nA0[k], nB0[k], ws + off, bytes, stream, &b->ctx[k]);
+    const size_t bytes = layout_of(&pk, split).total;
+    st = validate(&pk);
+    if (st == SC_OK && (!nA0[k] || !nB0[k])) st = fail(SC_EINVAL, "initial fields must be non-NULL");
+    if (st == SC_OK) st = create_context(&pk, nA0[k], nB0[k], ws + off, bytes, stream, split, &b->ctx[k]);
     if (st != SC_OK) {
       sc_batch_destroy(b);
       return st;
@@ -1461,7 +1485,7 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
   }
   // tables: per-lattice arguments (parity 0) and the block work list
   int nitems = 0;
-  batch_table_bytes(n, params, &nitems);
+  batch_table_bytes(n, params, split, &nitems);
   b->nitems = nitems;
   b->tile_y = b->ctx[0]->tile_y;
   b->args_dev = ws + off;
@@ -1473,7 +1497,7 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
   const int storage = params[0].storage;
   b->storage = storage;
   b->stencil = params[0].stencil == SC_FORCE_E6 ? kE6 : kE4;
-  b->split = batch_split(n, params) ? 1 : 0;
+  b->split = split ? 1 : 0;
   if (b->split) {
     b->sargs_dev = ws + off;
     b->sitems_dev = reinterpret_cast<int2 *>(ws + off + align_up(sizeof(SplitArgs<double>) * (size_t)n));

@@ -137,3 +137,53 @@ def test_fields_after_a_captured_step_are_computed_anew(B, L):
     for k in range(2):
         L.fake_reset()
         assert L.sc_moments(b.member(0), out[1], out[1], None) == B.SC_OK and fields_computed(L) == 1, k
+
+
+# bytes a site that the moments of the two-pass step need beyond the space of the FP64 fields
+GROWTH = [("F32", (0.0, 0.0), 0), ("F32", (-0.4, 0.0), 8), ("BF16", (0.0, 0.2), 8), ("F64", (0.0, 0.0), 32),
+          ("F64", (-0.4, 0.1), 48)]
+
+
+@pytest.mark.parametrize("storage,G_self,grown", GROWTH)
+def test_workspace_of_one_pass_is_enough(B, L, storage, G_self, grown):
+    """Only a context that steps in two passes asks for the room of the moments, and one that is given a workspace
+    without it steps in one pass; with less it is refused."""
+    shape, N = (32, 16, 16), 32 * 16 * 16
+    kw = dict(G=2.5, G_self=G_self, storage=getattr(B, f"SC_STORE_{storage}"))
+    size = lambda **more: B.sc_workspace_bytes(B.make_params(shape, **kw, **more))
+    one, two = size(variant=1), size()
+    assert two - one == grown * N and size(variant=2) == one and size(tau=(1.0, 0.9)) == one
+
+    def variant(c):
+        v = (ctypes.c_int32 * 8)()
+        assert L.sc_step_config(c.ctx, v, 8) == B.SC_OK
+        return v[0]
+
+    p = B.make_params(shape, **kw)
+    c = fake_gpu.Context(L, p)
+    assert c.status == B.SC_OK and variant(c) == 3
+    c = fake_gpu.Context(L, p, one)
+    assert c.status == B.SC_OK and variant(c) == (2 if grown else 3)
+    assert L.sc_step(c.ctx, 3) == B.SC_OK and c.moments() == B.SC_OK
+    assert fake_gpu.Context(L, p, one - 1).status == B.SC_ENOMEM
+    host, ws = fake_gpu.buffer(64 * N), fake_gpu.buffer(one)
+    h = [ctypes.c_void_p(host[1].value + 8 * N * k) for k in range(4)]
+    for nbytes, want in ((one, B.SC_OK), (one - 1, B.SC_ENOMEM)):
+        assert L.sc_run_host(ctypes.byref(p), h[0], h[1], 2, h[2], h[3], ws[1], nbytes, None) == want
+        assert L.sc_run_host_sigma(ctypes.byref(p), h[0], h[1], 2, None, 0.5, 4, h[2], h[3], host[1], ws[1], nbytes,
+                                   None) == want
+
+
+@pytest.mark.parametrize("storage,G_self,grown", GROWTH)
+def test_batch_workspace_of_one_pass_is_enough(B, L, storage, G_self, grown):
+    shapes = [(32, 16, 16), (40, 32, 8)]
+    kw = dict(G=2.5, G_self=G_self, storage=getattr(B, f"SC_STORE_{storage}"))
+    ps = [B.make_params(s, **kw) for s in shapes]
+    one = B.sc_batch_workspace_bytes([B.make_params(s, variant=2, **kw) for s in shapes])
+    two = B.sc_batch_workspace_bytes(ps)
+    assert two - one >= grown * sum(x * y * z for x, y, z in shapes)
+    assert L.sc_batch_variant(fake_gpu.Batch(L, ps).handle) == 4
+    b = fake_gpu.Batch(L, ps, one)
+    assert b.status == B.SC_OK and L.sc_batch_variant(b.handle) == 3
+    assert L.sc_batch_step(b.handle, 33) == B.SC_OK
+    assert fake_gpu.Batch(L, ps, one - 256).status == B.SC_ENOMEM
