@@ -39,7 +39,8 @@ LOCAL_REF_BYTES = {"f16": 16, "bf16": 16}
 # launch; reported only while the kernel sources still hash to the captured version.
 KERNEL_SOURCES = ["paper_2112_02574_gb300/csrc/sc_common.cuh", "paper_2112_02574_gb300/csrc/sc_step_kernel.cuh",
                   "paper_2112_02574_gb300/csrc/sc_step_staged.cuh", "paper_2112_02574_gb300/csrc/sc_step_split.cuh"]
-STEP_KERNELS = {1: "sc_step_kernel", 2: "sc_step_staged", 3: "sc_split_moments + sc_split_collide"}
+STEP_KERNELS = {1: "sc_step_kernel", 2: "sc_step_staged", 3: "sc_split_moments + sc_split_collide",
+                4: "sc_step_lanes"}
 # DRAM bytes per step launch (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture), keyed by the
 # kernel sources' hash, the storage and the launch (tile_y, stages, blocks_per_sm, blocks); a change to any of
 # them drops the figure (reported as null) until it is measured again

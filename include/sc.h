@@ -86,10 +86,10 @@ typedef struct {
                           eight waves of the GPU; either kernel 32 where that fills four,
                           else a balanced split whose grid fills whole waves; a batch: 64
                           staged, 32 generic; D2Q9: 1) */
-  int32_t variant;     /* step kernel: 0 = automatic (two passes or staged where they can run and are
-                          faster), 1 = generic (any size, any stencil), 2 = cp.async-staged (D3Q19, E4, nx >= 32
+  int32_t variant;     /* step kernel: 0 = automatic (two passes, staged, or for small D2Q9 lattices in FP64
+                          a thread per site and component, where they can run and are faster), 1 = generic (any size, any stencil), 2 = cp.async-staged (D3Q19, E4, nx >= 32
                           a multiple of the sites per 16-byte chunk: 1 F64, 2 F32, 4 F16 and
-                          BF16; tile_y 4, 8 or 16, F64 tile_y 4 only); both kernels compute
+                          BF16; tile_y 4, 8 or 16, F64 tile_y 4 only); all of them compute
                           the same numbers */
   int32_t stages;      /* staged kernel copy pipeline: 1 or 2 planes in flight; 0 = default */
   int32_t blocks_per_sm; /* staged kernel register budget: resident blocks per SM it must allow
@@ -370,7 +370,8 @@ int32_t sc_batch_active(const sc_batch *batch);
 void sc_batch_destroy(sc_batch *batch);
 
 /* The step kernel this context launches: out[0..8) = variant (1 generic, 2
- * staged, 3 two passes), tile_y, tile_z, stages, blocks_per_sm, blocks per launch
+ * staged, 3 two passes, 4 a thread per site and component: D2Q9 in FP64 up to 304
+ * blocks of 32 x 1 sites), tile_y, tile_z, stages, blocks_per_sm, blocks per launch
  * (of each pass), balanced split K (0: plain grid of tile_z chunks), columns with
  * K + 1 chunks; with two passes all but the blocks are 0.  n: room in out (>= 8).
  * Host only, no synchronisation. */

@@ -1722,7 +1722,7 @@ sc_status sc_step_config(const sc_ctx *c, int32_t *out, int32_t n) {
     for (int k = 0; k < 8; ++k) out[k] = v[k];
     return SC_OK;
   }
-  const int32_t v[8] = {c->staged ? 2 : 1, c->tile_y, c->tile_z, c->staged ? c->stages : 0,
+  const int32_t v[8] = {c->lanes ? 4 : (c->staged ? 2 : 1), c->tile_y, c->tile_z, c->staged ? c->stages : 0,
                         c->staged ? c->blocks_per_sm : 0, (int32_t)grid, c->zbal_k, c->zbal_rem};
   for (int k = 0; k < 8; ++k) out[k] = v[k];
   return SC_OK;

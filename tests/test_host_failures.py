@@ -187,3 +187,20 @@ def test_batch_workspace_of_one_pass_is_enough(B, L, storage, G_self, grown):
     assert b.status == B.SC_OK and L.sc_batch_variant(b.handle) == 3
     assert L.sc_batch_step(b.handle, 33) == B.SC_OK
     assert fake_gpu.Batch(L, ps, one - 256).status == B.SC_ENOMEM
+
+
+@pytest.mark.parametrize("shape,more,want", [
+    ((64, 64, 1), {}, (4, 1, 128)),                   # a thread per site and component: blocks of 32 x 1 sites
+    ((64, 64, 1), dict(tile_y=1), (1, 1, 128)),       # the same tile asked for: the generic kernel
+    ((64, 64, 1), dict(variant=1), (1, 4, 32)),
+    ((512, 512, 1), {}, (1, 4, 2048)),
+    ((64, 64, 1), dict(storage=0), (1, 4, 32)),
+])
+def test_step_config_names_the_small_d2q9_kernel(B, L, shape, more, want):
+    c = fake_gpu.Context(L, B.make_params(shape, **{**dict(lattice=B.SC_D2Q9, storage=B.SC_STORE_F64, G=2.5), **more}))
+    v = (ctypes.c_int32 * 8)()
+    assert L.sc_step_config(c.ctx, v, 8) == B.SC_OK
+    assert (v[0], v[1], v[5]) == want
+    L.fake_reset()
+    assert L.sc_step(c.ctx, 1) == B.SC_OK
+    assert [("lanes" in n) for n in fake_gpu.calls(L)] == [want[0] == 4]
