@@ -318,7 +318,7 @@ struct sc_batch {
   size_t smem;
   // the two-pass form: SplitArgs<CT>[n], (lattice, first site) per block, and the groups of members that step
   // together (group g: items group_at[g] .. group_at[g + 1] - 1)
-  int split, nsplit, stencil, storage;
+  int split, stencil, storage;
   int *group_at, ngroups;
   int *group_one;  // the member of a group of one large lattice (launched as a lone lattice is), else -1
   void *sargs_dev;
@@ -1186,11 +1186,10 @@ bool batch_split(int32_t n, const sc_params *params) {
 // 8 droplets (1.9 M) FP32 108.5 -> 99.4; 16 droplets (22.1 M, mostly large members) FP32 1234 -> 1225, FP16 1006 -> 994.
 constexpr int64_t kGroupSites = 768 << 10;
 // Its tables: SplitArgs of the members, then the items.
-size_t split_table_bytes(int32_t n, const sc_params *params, int64_t *items_out) {
+size_t split_table_bytes(int32_t n, const sc_params *params) {
   int64_t items = 0;
   for (int k = 0; k < n; ++k)
     items += ((int64_t)params[k].nx * params[k].ny * params[k].nz + kSplitBatchSites - 1) / kSplitBatchSites;
-  if (items_out) *items_out = items;
   return align_up(sizeof(SplitArgs<double>) * (size_t)n) + align_up(sizeof(int2) * (size_t)items);
 }
 
@@ -1204,7 +1203,7 @@ size_t batch_table_bytes(int32_t n, const sc_params *params, bool split, int *ni
   }
   if (nitems_out) *nitems_out = nitems;
   return align_up(sizeof(StepArgs<double>) * (size_t)n) + align_up(sizeof(int4) * (size_t)nitems) + kAlign +
-         (split ? split_table_bytes(n, params, nullptr) : 0);
+         (split ? split_table_bytes(n, params) : 0);
 }
 
 // Workspace of a batch that steps in two passes, or does not.
@@ -1250,7 +1249,6 @@ sc_status batch_upload_items(sc_batch *b) {
     total += ((c->p.nx + 31) / 32) * ((c->p.ny + c->tile_y - 1) / c->tile_y) * ((c->p.nz + c->tile_z - 1) / c->tile_z);
   }
   b->nitems = total;
-  b->nsplit = 0;
   if (total == 0) return SC_OK;
   if (b->sitems_dev) {
     int64_t count = 0;
@@ -1281,7 +1279,6 @@ sc_status batch_upload_items(sc_batch *b) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     delete[] si;
     if (e != cudaSuccess) return fail(SC_ECUDA, "uploading the batch work list: %s", cudaGetErrorString(e));
-    b->nsplit = (int)count;
   }
   int4 *items = new (std::nothrow) int4[total];
   if (!items) return fail(SC_ENOMEM, "host allocation failed");

@@ -11,9 +11,10 @@ cudaError_t launch_split(int sten, const SplitArgs<CT> &m, cudaStream_t st) {
   const unsigned blocks = (unsigned)((m.a.N + kSplitThreads - 1) / kSplitThreads);
   cudaError_t e = launch_pass(sc_split_moments<ST, CT>, blocks, kSplitThreads, 0, st, m);
   if (e != cudaSuccess) return e;
-  const bool small = sizeof(CT) == 4 && m.a.self_on && m.a.N <= kSmallCollide;
-  auto *collide = sten == kE6 ? (small ? sc_split_collide<kE6, ST, CT, true> : sc_split_collide<kE6, ST, CT, false>)
-                              : (small ? sc_split_collide<kE4, ST, CT, true> : sc_split_collide<kE4, ST, CT, false>);
+  auto *collide = sten == kE6 ? sc_split_collide<kE6, ST, CT, false> : sc_split_collide<kE4, ST, CT, false>;
+  if constexpr (sizeof(CT) == 4)  // FP64 has one register budget
+    if (m.a.self_on && m.a.N <= kSmallCollide)
+      collide = sten == kE6 ? sc_split_collide<kE6, ST, CT, true> : sc_split_collide<kE4, ST, CT, true>;
   return launch_pass(collide, blocks, kSplitThreads, 0, st, m);
 }
 
