@@ -111,12 +111,13 @@ __global__ void pop_kernel(PopArgs a, int mode, const double *n0A, const double 
   }
 }
 
-// Exact-to-FP64 sums of FP32 pairs.  GB300 issues one FP64 warp instruction per 16 cycles and SM but four FP32
+// Sums of FP32 pairs to FP64 accuracy.  GB300 issues one FP64 warp instruction per 16 cycles and SM but four FP32
 // ones per cycle, so sums of values that are stored in FP32 (or fewer bits) are kept as three FP32 terms: each
-// addition is Knuth's TwoSum (an error-free transformation) with the error passed down, so that what is dropped is
-// below 2^-70 of the sum, and only the result is converted.  Against FP64 sums of the 38 populations of a site
-// (38 conversions, 38 additions): density fields of 128^3 FP32 647 -> 88 us, BF16 with one psi 1062 -> 197 us,
-// velocity BF16 1929 -> 683 us (its force stays FP64).
+// addition is Knuth's TwoSum (an error-free transformation) with the error passed down, and only the result is
+// converted.  Nothing is lost but the roundings of the third term: for n terms at most n^3 2^-72 of the sum of their
+// magnitudes, 2^-59 for the 19 of a density, against the 2^-53 of each FP64 addition.  A sum beyond the FP32 range is infinite.
+// Against FP64 sums of the 38 populations of a site (38 conversions, 38 additions): density fields of 128^3 FP32
+// 647 -> 88 us, BF16 with one psi 1062 -> 197 us, velocity BF16 1929 -> 683 us (its force stays FP64).
 struct PairSum3 {
   float2 a = {0.0f, 0.0f}, b = {0.0f, 0.0f}, c = {0.0f, 0.0f};
   __device__ __forceinline__ static float2 neg_add(float2 x, float2 y) {  // x - y
@@ -130,9 +131,12 @@ struct PairSum3 {
   }
   __device__ __forceinline__ void add(float2 v) { c = __fadd2_rn(c, two_sum(b, two_sum(a, v))); }
   __device__ __forceinline__ void sub(float2 v) { add(make_float2(-v.x, -v.y)); }
-  __device__ __forceinline__ double2 value() const {
-    return make_double2(((double)c.x + (double)b.x) + (double)a.x, ((double)c.y + (double)b.y) + (double)a.y);
+  // An infinite or NaN term leaves inf - inf in the errors, so the leading term, once it is not finite, is the sum.
+  __device__ __forceinline__ static double total(float a, float b, float c) {
+    const double s = ((double)c + (double)b) + (double)a;
+    return (__float_as_uint(a) & 0x7f800000u) == 0x7f800000u ? (double)a : s;
   }
+  __device__ __forceinline__ double2 value() const { return make_double2(total(a.x, b.x, c.x), total(a.y, b.y, c.y)); }
 };
 struct PairSumD {
   double2 s = {0.0, 0.0};
