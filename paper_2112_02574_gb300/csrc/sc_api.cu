@@ -960,7 +960,8 @@ sc_status sc_sigma_minimum(const double *rows, int32_t nbins, const double *P_in
   if (dim != 2 && dim != 3) return fail(SC_EINVAL, "dim must be 2 or 3");
   if (!(R_lo > 0.0) || !(R_hi > R_lo) || !(R_step > 0.0) || (R_hi - R_lo) / R_step > 1e7)
     return fail(SC_EINVAL, "need 0 < R_lo < R_hi, R_step > 0 and at most 1e7 grid points");
-  sigma_kernel<<<1, kSigmaThreads, 0, static_cast<cudaStream_t>(stream)>>>(rows, nbins, P_in_out, dim, R_lo, R_hi, R_step, out);
+  const int threads = nbins <= 32 && (R_hi - R_lo) / R_step < 31.0 ? 32 : kSigmaThreads;
+  sigma_kernel<<<1, threads, 0, static_cast<cudaStream_t>(stream)>>>(rows, nbins, P_in_out, dim, R_lo, R_hi, R_step, out);
   SC_CUDA(cudaGetLastError());
   return SC_OK;
 }

@@ -447,24 +447,26 @@ __global__ void bulk_pressure_kernel(ForceParams fp, const double *fields, int64
   out[threadIdx.x] = P;
 }
 
-// sigma[R] minimum (section 3) on one block of 256 threads; see sc_sigma_minimum in sc.h.
+// sigma[R] minimum (section 3) on one block of 256 threads (one warp for at most 32 rows and samples); see sc_sigma_minimum in sc.h.
 //  * The trapezoid of r^(dim-1) P_T: rows come 256 at a time into shared memory, every thread forms the term of its
 //    row with the last non-empty row before it, and the terms are added in a fixed tree.
 //  * The grid search needs sigma[R] in FP64 only where it can be the minimum: FP32 values of all samples, good to
 //    1e-5 of the sizes of their two terms, leave those whose lower bound is below every upper bound.
-// One warp did both one after another before: 212 us at 128 rows and 6400 samples, now 18 us.
+// One warp did both one after another before: 212 us at 128 rows and 6400 samples, now 18 us.  The trees and the
+// search for a chunk's last row span the rows and samples there are: 2 rows and 5 samples 18.9 -> 11.3 us (9.8 in the
+// one warp).
 constexpr int kSigmaThreads = 256;
 __global__ void __launch_bounds__(kSigmaThreads) sigma_kernel(const double *rows, int nbins, const double *pio, int dim,
                                                               double R_lo, double R_hi, double R_step, double *out) {
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, nt = blockDim.x;
   __shared__ double s_r[kSigmaThreads], s_f[kSigmaThreads], s_t[kSigmaThreads];
   __shared__ int s_on[kSigmaThreads];
   __shared__ int s_i[kSigmaThreads];
   __shared__ float s_u[kSigmaThreads];
   double T = 0.0, rp = 0.0, fp = 0.0;  // rp, fp: the last non-empty row of the chunks before
   bool any = false;
-  for (int b0 = 0; b0 < nbins; b0 += kSigmaThreads) {
-    const int b = b0 + tid;
+  for (int b0 = 0; b0 < nbins; b0 += nt) {
+    const int b = b0 + tid, rows_here = min(nt, nbins - b0);
     const bool on = b < nbins && rows[b * 6 + 5] > 0.0;
     const double r = on ? rows[b * 6 + 0] : 0.0, pt = on ? rows[b * 6 + 2] : 0.0;
     const double f = (dim == 3 ? r * r : r) * pt;
@@ -482,7 +484,7 @@ __global__ void __launch_bounds__(kSigmaThreads) sigma_kernel(const double *rows
         term = 0.5 * (f + fp) * (r - rp);
     }
     s_t[tid] = term;
-    int last = kSigmaThreads - 1;
+    int last = rows_here - 1;
     while (last >= 0 && !s_on[last]) --last;
     if (last >= 0) {
       rp = s_r[last];
@@ -490,7 +492,7 @@ __global__ void __launch_bounds__(kSigmaThreads) sigma_kernel(const double *rows
       any = true;
     }
     __syncthreads();
-    for (int w = kSigmaThreads / 2; w > 0; w >>= 1) {
+    for (int w = tree_top(rows_here); w > 0; w >>= 1) {
       if (tid < w) s_t[tid] += s_t[tid + w];
       __syncthreads();
     }
@@ -509,23 +511,25 @@ __global__ void __launch_bounds__(kSigmaThreads) sigma_kernel(const double *rows
     up = u + v + m;
   };
   float best_up = INFINITY;
-  for (int k = tid; k < ng; k += kSigmaThreads) {
-    float down, up;
-    bounds(k, down, up);
-    best_up = fminf(best_up, up);  // a NaN bound is ignored here and its sample kept below
-  }
-  s_u[tid] = best_up;
-  __syncthreads();
-  for (int w = kSigmaThreads / 2; w > 0; w >>= 1) {
-    if (tid < w) s_u[tid] = fminf(s_u[tid], s_u[tid + w]);
-    __syncthreads();
-  }
-  // sizes outside FP32's comfortable range: every sample in FP64
+  // a warp's worth of samples, or sizes outside FP32's comfortable range: every sample in FP64
   const double big = fmax(fabs(dP), fabs(C)), small = fmin(fabs(dP), fabs(C));
-  best_up = (big < 1e25 && small > 1e-25 && R_lo > 1e-4 && R_hi < 1e8) ? s_u[0] : INFINITY;
+  if (ng > 32 && big < 1e25 && small > 1e-25 && R_lo > 1e-4 && R_hi < 1e8) {
+    for (int k = tid; k < ng; k += nt) {
+      float down, up;
+      bounds(k, down, up);
+      best_up = fminf(best_up, up);  // a NaN bound is ignored here and its sample kept below
+    }
+    s_u[tid] = best_up;
+    __syncthreads();
+    for (int w = tree_top(min(ng, nt)); w > 0; w >>= 1) {
+      if (tid < w) s_u[tid] = fminf(s_u[tid], s_u[tid + w]);
+      __syncthreads();
+    }
+    best_up = s_u[0];
+  }
   double best = INFINITY;
   int bi = -1;
-  for (int k = tid; k < ng; k += kSigmaThreads) {
+  for (int k = tid; k < ng; k += nt) {
     float down, up;
     bounds(k, down, up);
     if (down > best_up && down < INFINITY) continue;
@@ -538,7 +542,7 @@ __global__ void __launch_bounds__(kSigmaThreads) sigma_kernel(const double *rows
   s_t[tid] = best;
   s_i[tid] = bi;
   __syncthreads();
-  for (int w = kSigmaThreads / 2; w > 0; w >>= 1) {
+  for (int w = tree_top(min(ng, nt)); w > 0; w >>= 1) {
     if (tid < w) {
       const double ob = s_t[tid + w];
       const int oi = s_i[tid + w];
