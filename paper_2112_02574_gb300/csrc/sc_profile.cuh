@@ -264,6 +264,11 @@ __global__ void __launch_bounds__(256) profile_partial_kernel(ForceParams fp, Pr
   __syncthreads();
   double *out = partial + (int64_t)blockIdx.x * row;
   const double *all = reinterpret_cast<const double *>(smem_raw);
+  if (nwarps == 1) {  // many bins: a plain copy, whose loads the loop overlaps
+#pragma unroll 8
+    for (int k = lane; k < row; k += 32) out[k] = all[k];
+    return;
+  }
   for (int k = threadIdx.x; k < row; k += blockDim.x) {
     double acc = all[k];
     for (int w = 1; w < nwarps; ++w) acc += all[(int64_t)w * (row + 32 * 5) + k];
@@ -288,6 +293,26 @@ __global__ void __launch_bounds__(192) profile_finalize_kernel(const T *partial,
   if (lane == 0) sum[c] = red[c][0];
   __syncthreads();
   if (lane == 0) out[b * 6 + c] = c == 5 ? sum[5] : (sum[5] > 0 ? sum[c] / sum[5] : 0.0);
+}
+
+// The same means, the same order of additions, with a thread per bin and component (a block: 32 bins), for many bins
+// of few blocks (at most 32), where a block per bin is mostly launch: 8^3 sites in 4096 bins 54.7 -> 29.0 us (39.1 with a thread per bin and a slower copy of the bins).
+template <class T>
+__global__ void __launch_bounds__(192) profile_finalize_few_kernel(const T *partial, int nblocks, int nbins, T *out) {
+  __shared__ T sum[192];
+  const int at = blockIdx.x * 192 + threadIdx.x, n = nbins * 6, c = threadIdx.x % 6;
+  T v[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) v[k] = k < nblocks && at < n ? T(0.0) + partial[(int64_t)k * n + at] : T(0.0);
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+    for (int k = 0; k < w; ++k)
+      if (k + w < nblocks) v[k] += v[k + w];
+  sum[threadIdx.x] = v[0];
+  __syncthreads();
+  const T count = sum[threadIdx.x - c + 5];
+  if (at < n) out[at] = c == 5 ? count : (count > 0 ? v[0] / count : T(0.0));
 }
 
 // Blocks of a profile launch and the sites each one takes (a multiple of 32):
@@ -330,7 +355,10 @@ cudaError_t launch_profile_kind(const ForceParams &fp, ProfileArgs pa, const FA 
   k<<<(int)blocks, 32 * warps, smem, st>>>(fp, pa, fld, tables, partial);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  profile_finalize_kernel<double><<<pa.nbins, 192, 0, st>>>(partial, (int)blocks, pa.nbins, out);
+  if (blocks <= 32 && pa.nbins >= 1024)
+    profile_finalize_few_kernel<double><<<(pa.nbins + 31) / 32, 192, 0, st>>>(partial, (int)blocks, pa.nbins, out);
+  else
+    profile_finalize_kernel<double><<<pa.nbins, 192, 0, st>>>(partial, (int)blocks, pa.nbins, out);
   return cudaGetLastError();
 }
 
