@@ -46,22 +46,45 @@ cudaError_t launch_pass(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem
   return cudaLaunchKernelEx(&c, kernel, args...);
 }
 
+// D2Q9 lattices up to this many sites step as programmatic dependents.  The plain loads that these need cost the
+// tau = 1 kernels registers (FP32 84 -> 102, BF16 96 -> 118: four blocks per SM, not five), which from here on is more
+// than the launch latency saved.  Plain launches -> dependents, us a step: FP32 256^2 3.16 -> 2.95, 384^2 4.99 -> 4.92, 448^2
+// 6.15 -> 6.39, 1024^2 31.0 -> 34.0; BF16 384^2 5.51 -> 5.38, 448^2 6.94 -> 6.99, 1024^2 30.3 -> 32.9; FP16 (four blocks
+// either way) 640^2 12.90 -> 12.81, 1024^2 33.30 -> 33.38, 2048^2 127.7 -> 128.3.  FP64 and tau != 1 gain at every size.
+template <class ST, class CT>
+bool dependent_d2q9(const StepArgs<CT> &a) {
+  if (sizeof(CT) == 8 || !a.tau_one) return true;
+  return a.N <= (std::is_same<ST, __half>::value ? 800000 : 180000);
+}
+
 // T1 selects the tau_A = tau_B = 1 instantiation (StepArgs::tau_one).
 template <int LAT, int STEN, class ST, class CT, int TY>
 cudaError_t launch_one(const StepLaunch &l, const StepArgs<CT> &a) {
   constexpr size_t smem = step_smem_bytes<LAT, STEN, CT, TY>();
-  auto *k = a.tau_one ? sc_step_kernel<LAT, STEN, ST, CT, TY, true> : sc_step_kernel<LAT, STEN, ST, CT, TY, false>;
-  if (!attr_once(reinterpret_cast<const void *>(k), smem)) return cudaGetLastError();
   const dim3 grid = a.zbal_k > 0 ? dim3(a.zbal_k * a.zbal_cols + a.zbal_rem) : l.grid;
-  if constexpr (LAT == kD2Q9) return launch_pass(k, grid, dim3(32, TY), smem, l.stream, a);
-  k<<<grid, dim3(32, TY), smem, l.stream>>>(a);
+  if constexpr (LAT == kD2Q9) {
+    if (dependent_d2q9<ST, CT>(a)) {
+      auto *k = a.tau_one ? sc_step_kernel<LAT, STEN, ST, CT, TY, true, true>
+                          : sc_step_kernel<LAT, STEN, ST, CT, TY, false, true>;
+      if (!attr_once(reinterpret_cast<const void *>(k), smem)) return cudaGetLastError();
+      return launch_pass(k, grid, dim3(32, TY), smem, l.stream, a);
+    }
+  }
+  if constexpr (LAT == kD3Q19 || sizeof(CT) == 4) {
+    auto *k = sc_step_kernel<LAT, STEN, ST, CT, TY, true, false>;
+    if constexpr (LAT == kD3Q19)
+      if (!a.tau_one) k = sc_step_kernel<LAT, STEN, ST, CT, TY, false, false>;
+    if (!attr_once(reinterpret_cast<const void *>(k), smem)) return cudaGetLastError();
+    k<<<grid, dim3(32, TY), smem, l.stream>>>(a);
+  }
   return cudaGetLastError();
 }
 
 template <int LAT, int STEN, class ST, class CT, int TY>
 cudaError_t generic_occupancy_one(bool t1, int *blocks) {
   constexpr size_t smem = step_smem_bytes<LAT, STEN, CT, TY>();
-  auto *k = t1 ? sc_step_kernel<LAT, STEN, ST, CT, TY, true> : sc_step_kernel<LAT, STEN, ST, CT, TY, false>;
+  constexpr bool DEP = LAT == kD2Q9;
+  auto *k = t1 ? sc_step_kernel<LAT, STEN, ST, CT, TY, true, DEP> : sc_step_kernel<LAT, STEN, ST, CT, TY, false, DEP>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, 32 * TY, smem);

@@ -43,8 +43,9 @@ __device__ __forceinline__ P2<CT> unscale(P2<CT> v, P2<CT> inv_scale) {
 // Pull the Q population pairs arriving at site (gx, gy, gz) and return their
 // sum (the density deviations, natural units); values go to v[] (step units) when
 // V is true.  Values are deviations from w_i nbar; with a local reference the source
-// site's density deviation nsrc[s] = n(s) - nbar enters as w_i nsrc[s].
-template <int LAT, class ST, class CT, bool V>
+// site's density deviation nsrc[s] = n(s) - nbar enters as w_i nsrc[s].  DEP: the kernel is a
+// programmatic dependent (see pass_begin), so the loads are plain ones.
+template <int LAT, class ST, class CT, bool V, bool DEP>
 __device__ __forceinline__ P2<CT> pull_site(const ST *__restrict__ src, int gx, int gy, int gz, int nx, int ny,
                                             int nz, int64_t N, P2<CT> scale, P2<CT> inv_scale, P2<CT> *v,
                                             const float2 *__restrict__ nsrc = nullptr) {
@@ -58,10 +59,9 @@ __device__ __forceinline__ P2<CT> pull_site(const ST *__restrict__ src, int gx, 
   for (int i = 0; i < L::Q; ++i) {
     const int cx = L::c(i, 0), cy = L::c(i, 1), cz = L::c(i, 2);
     const int site = X[cx + 1] + nx * (Y[cy + 1] + ny * Z[cz + 1]);
-    // D2Q9 launches are programmatic dependents (see pass_begin): plain loads
-    P2<CT> g = Codec2<ST, CT>::template load<LAT == kD2Q9>(src + ((int64_t)i * N + site) * 2, inv_scale);
+    P2<CT> g = Codec2<ST, CT>::template load<DEP>(src + ((int64_t)i * N + site) * 2, inv_scale);
     if constexpr (local_ref<ST>()) {
-      const float2 ns = LAT == kD2Q9 ? nsrc[site] : __ldg(nsrc + site);
+      const float2 ns = DEP ? nsrc[site] : __ldg(nsrc + site);
       g = pfma(wpair<LAT, ST, CT>(i, scale), pset(CT(ns.x), CT(ns.y)), g);
     }
     if (V) v[i] = g;
@@ -378,7 +378,7 @@ __device__ __forceinline__ void block_work(const StepArgs<CT> &a, int &bx, int &
 
 // One block's work: the column (bx, by), planes z0 .. zend - 1, of the lattice described by a,
 // marched upward or (down) downward.
-template <int LAT, int STEN, class ST, class CT, int TY, bool T1>
+template <int LAT, int STEN, class ST, class CT, int TY, bool T1, bool DEP>
 __device__ __forceinline__ void step_block(const StepArgs<CT> &a, int bx, int by, int z0, int zend, bool down,
                                            unsigned char *smem_raw) {
   using L = Lattice<LAT>;
@@ -436,9 +436,9 @@ __device__ __forceinline__ void step_block(const StepArgs<CT> &a, int bx, int by
       const int idx = (py + H) * SX + (px + H);
       P2<CT> g[Q];
       const P2<CT> dn =
-          pull_site<LAT, ST, CT, KEEP>(src, gx, gy, gz, nx, ny, nz, N, a.scale, a.inv_scale, g, a.nsrc);
+          pull_site<LAT, ST, CT, KEEP, DEP>(src, gx, gy, gz, nx, ny, nz, N, a.scale, a.inv_scale, g, a.nsrc);
       const P2<CT> dh =
-          pull_site<LAT, ST, CT, false>(src, hx, hy, gz, nx, ny, nz, N, a.scale, a.inv_scale, nullptr, a.nsrc);
+          pull_site<LAT, ST, CT, false, DEP>(src, hx, hy, gz, nx, ny, nz, N, a.scale, a.inv_scale, nullptr, a.nsrc);
       s_dn[slot * PLANE + own] = dn;
       if (hal) s_dn[slot * PLANE + idx] = dh;
       if (a.self_on) {
@@ -459,7 +459,7 @@ __device__ __forceinline__ void step_block(const StepArgs<CT> &a, int bx, int by
       {
         P2<CT> g[Q];
         const P2<CT> dn =
-            pull_site<LAT, ST, CT, KEEP>(src, gx, gy, gz, nx, ny, nz, N, a.scale, a.inv_scale, g, a.nsrc);
+            pull_site<LAT, ST, CT, KEEP, DEP>(src, gx, gy, gz, nx, ny, nz, N, a.scale, a.inv_scale, g, a.nsrc);
         s_dn[slot * PLANE + own] = dn;
         if (a.self_on) s_psi[slot * PLANE + own] = psi_deviation<CT>(dn, a.nbar, a.psibar, a.psi_exp, a.gself);
         if constexpr (KEEP) {
@@ -484,7 +484,7 @@ __device__ __forceinline__ void step_block(const StepArgs<CT> &a, int bx, int by
         }
         const int hx = ((x0 + px) % nx + nx) % nx, hy = ((y0 + py) % ny + ny) % ny;
         const P2<CT> dn =
-            pull_site<LAT, ST, CT, false>(src, hx, hy, gz, nx, ny, nz, N, a.scale, a.inv_scale, nullptr, a.nsrc);
+            pull_site<LAT, ST, CT, false, DEP>(src, hx, hy, gz, nx, ny, nz, N, a.scale, a.inv_scale, nullptr, a.nsrc);
         const int idx = (py + H) * SX + (px + H);
         s_dn[slot * PLANE + idx] = dn;
         if (a.self_on) s_psi[slot * PLANE + idx] = psi_deviation<CT>(dn, a.nbar, a.psibar, a.psi_exp, a.gself);
@@ -513,7 +513,7 @@ __device__ __forceinline__ void step_block(const StepArgs<CT> &a, int bx, int by
         collide_site<LAT, STEN, ST, CT, TY, T1>(a, car[0], s_dn, s_psi, sl, own, valid_xy, dst, site);
       } else {
         P2<CT> g[Q];
-        pull_site<LAT, ST, CT, true>(src, gx, gy, gzc, nx, ny, nz, N, a.scale, a.inv_scale, g, a.nsrc);
+        pull_site<LAT, ST, CT, true, DEP>(src, gx, gy, gzc, nx, ny, nz, N, a.scale, a.inv_scale, g, a.nsrc);
         collide_site<LAT, STEN, ST, CT, TY, T1>(a, g, s_dn, s_psi, sl, own, valid_xy, dst, site);
       }
     }
@@ -521,15 +521,15 @@ __device__ __forceinline__ void step_block(const StepArgs<CT> &a, int bx, int by
   }
 }
 
-// T1: the tau_A = tau_B = 1 form (see carry_size).
-template <int LAT, int STEN, class ST, class CT, int TY, bool T1>
+// T1: the tau_A = tau_B = 1 form (see carry_size).  DEP: launched as a programmatic dependent.
+template <int LAT, int STEN, class ST, class CT, int TY, bool T1, bool DEP>
 __global__ void __launch_bounds__(32 * TY, (TY >= 16 ? 1 : 16 / TY)) sc_step_kernel(const StepArgs<CT> a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   int bx, by, z0, zend;
   bool down;
   block_work(a, bx, by, z0, zend, down);
-  if constexpr (LAT == kD2Q9) pass_begin();
-  step_block<LAT, STEN, ST, CT, TY, T1>(a, bx, by, z0, zend, down, smem_raw);
+  if constexpr (DEP) pass_begin();
+  step_block<LAT, STEN, ST, CT, TY, T1, DEP>(a, bx, by, z0, zend, down, smem_raw);
 }
 
 // Batched form: one launch steps several lattices.  Block b works on item
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(32 * TY, (TY >= 16 ? 1 : 16 / TY))
     a.ndst = const_cast<float2 *>(u);
   }
   const int z0 = it.w * a.tile_z;
-  step_block<LAT, STEN, ST, CT, TY, T1>(a, it.y, it.z, z0, min(z0 + a.tile_z, a.nz), false, smem_raw);
+  step_block<LAT, STEN, ST, CT, TY, T1, false>(a, it.y, it.z, z0, min(z0 + a.tile_z, a.nz), false, smem_raw);
 }
 
 }  // namespace scgb

@@ -1,6 +1,7 @@
 /* A CUDA runtime without a GPU, for tests of the library's host logic: device memory is host memory, copies and
  * memsets are done, kernels are recorded by name and not run, and the n-th call of a chosen kind can be made to
- * fail.  The library's objects are linked with this file instead of the CUDA runtime. */
+ * fail.  Asynchronous copies to the host deliver doubles of 1 (valid densities) in place of what the kernels would have
+ * written.  The library's objects are linked with this file instead of the CUDA runtime. */
 #include <cuda_runtime_api.h>
 #include <stdio.h>
 #include <string.h>
@@ -8,6 +9,7 @@
 enum { MAX_FUNCS = 4096, MAX_LOG = 1 << 16 };
 static const void *g_fun[MAX_FUNCS];
 static char g_name[MAX_FUNCS][192];
+static char g_dep[MAX_FUNCS][208]; /* the same, launched as a programmatic dependent */
 static int g_nfun;
 
 /* Recorded calls: kernel names, and "graph launch". */
@@ -36,12 +38,12 @@ static cudaError_t result(const char *what) {
 static void record(const char *s) {
   if (g_nlog < MAX_LOG) g_log[g_nlog++] = s;
 }
-static cudaError_t launch(const void *f) {
+static cudaError_t launch(const void *f, int dep) {
   const cudaError_t e = result("kernel");
   if (e != cudaSuccess) return e;
   for (int k = 0; k < g_nfun; ++k)
     if (g_fun[k] == f) {
-      record(g_name[k]);
+      record(dep ? g_dep[k] : g_name[k]);
       return cudaSuccess;
     }
   return (cudaError_t)(g_last = cudaErrorInvalidDeviceFunction);
@@ -56,7 +58,9 @@ void __cudaRegisterFunction(void **h, const char *host, char *dev, const char *n
   (void)h, (void)dev, (void)limit, (void)tid, (void)bid, (void)bd, (void)gd, (void)ws;
   if (g_nfun == MAX_FUNCS) return;
   g_fun[g_nfun] = host;
-  snprintf(g_name[g_nfun++], sizeof g_name[0], "%s", name);
+  snprintf(g_name[g_nfun], sizeof g_name[0], "%s", name);
+  snprintf(g_dep[g_nfun], sizeof g_dep[0], "%s (dependent)", g_name[g_nfun]);
+  g_nfun++;
 }
 void __cudaRegisterVar(void **h, char *host, char *dev, const char *name, int ext, size_t size, int c, int g) {
   (void)h, (void)host, (void)dev, (void)name, (void)ext, (void)size, (void)c, (void)g;
@@ -76,15 +80,15 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
 }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **args, size_t smem, cudaStream_t st) {
   (void)g, (void)b, (void)args, (void)smem, (void)st;
-  return launch((const void *)k);
+  return launch((const void *)k, 0);
 }
 
 cudaError_t cudaLaunchKernel(const void *f, dim3 g, dim3 b, void **args, size_t smem, cudaStream_t st) {
   return __cudaLaunchKernel((cudaKernel_t)f, g, b, args, smem, st);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) {
-  (void)c, (void)args;
-  return launch(f);
+  (void)args;
+  return launch(f, c->numAttrs > 0);
 }
 cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, enum cudaDeviceAttr a, int d) {
@@ -111,7 +115,9 @@ cudaError_t cudaMemcpy(void *d, const void *s, size_t n, enum cudaMemcpyKind k) 
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, enum cudaMemcpyKind k, cudaStream_t st) {
   (void)st;
   const cudaError_t e = result("cudaMemcpyAsync");
-  return e == cudaSuccess ? cudaMemcpy(d, s, n, k) : e;
+  if (e != cudaSuccess || k != cudaMemcpyDeviceToHost) return e == cudaSuccess ? cudaMemcpy(d, s, n, k) : e;
+  for (size_t i = 0; i < n / sizeof(double); ++i) ((double *)d)[i] = 1.0;
+  return cudaSuccess;
 }
 cudaError_t cudaMemset(void *d, int v, size_t n) { return memset(d, v, n), cudaSuccess; }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t st) { return (void)st, cudaMemset(d, v, n); }
@@ -136,7 +142,7 @@ cudaError_t cudaGraphAddKernelNode(cudaGraphNode_t *n, cudaGraph_t g, const cuda
                                    const struct cudaKernelNodeParams *p) {
   (void)g, (void)d, (void)nd;
   *n = (cudaGraphNode_t)1;
-  return launch(p->func);
+  return launch(p->func, 0);
 }
 cudaError_t cudaGraphAddMemsetNode(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *d, size_t nd,
                                    const struct cudaMemsetParams *p) {

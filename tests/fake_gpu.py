@@ -1,11 +1,13 @@
 """The library linked with fake_cudart.c: its host logic on a machine without a GPU, with failures at chosen calls."""
 import ctypes
 import importlib
+import mmap
 import os
 import subprocess
 
 import numpy as np
 
+MAP_NORESERVE = 0x4000  # of Linux; not in the mmap module
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 
@@ -36,10 +38,9 @@ def calls(L):
 
 
 def buffer(nbytes):
-    """"Device" memory: 256-byte aligned, every double in it 1 (so that unrun reductions give valid densities)."""
-    a = np.ones(nbytes // 8 + 64)
-    off = -a.ctypes.data % 256
-    v = a.view(np.uint8)[off:off + nbytes]
+    """"Device" memory, page aligned; pages that nothing touches take no memory."""
+    m = mmap.mmap(-1, nbytes, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS | MAP_NORESERVE)
+    v = np.frombuffer(m, dtype=np.uint8)
     return v, ctypes.c_void_p(v.ctypes.data)
 
 

@@ -204,3 +204,14 @@ def test_step_config_names_the_small_d2q9_kernel(B, L, shape, more, want):
     L.fake_reset()
     assert L.sc_step(c.ctx, 1) == B.SC_OK
     assert [("lanes" in n) for n in fake_gpu.calls(L)] == [want[0] == 4]
+
+
+@pytest.mark.parametrize("storage,tau,side,dependent", [
+    ("F32", 1.0, 424, True), ("F32", 1.0, 425, False), ("BF16", 1.0, 424, True), ("BF16", 1.0, 425, False),
+    ("F16", 1.0, 894, True), ("F16", 1.0, 895, False), ("F32", 0.9, 1024, True), ("F64", 1.0, 1024, True)])
+def test_large_d2q9_lattices_take_plain_launches(B, L, storage, tau, side, dependent):
+    c = fake_gpu.Context(L, B.make_params((side, side, 1), lattice=B.SC_D2Q9, tau=(tau, tau), G=2.5,
+                                          storage=getattr(B, f"SC_STORE_{storage}")))
+    L.fake_reset()
+    assert L.sc_step(c.ctx, 1) == B.SC_OK
+    assert [n.endswith("(dependent)") for n in fake_gpu.calls(L)] == [dependent]
