@@ -286,12 +286,14 @@ __device__ __forceinline__ void collide_pair(const StepArgs<CT> &a, const P2<CT>
   }
 }
 
-// Status: a non-finite density, or a non-positive one while psi = exp(-1/n) is in use.
-template <class CT>
+// Status: a non-finite density, or a non-positive one while psi = exp(-1/n) is in use.  LOOK: the word is read first
+// and set once (an atomic per site of a lattice that has failed everywhere costs the collision pass more than its work).
+template <class CT, bool LOOK = false>
 __device__ __forceinline__ void check_density(const StepArgs<CT> &a, P2<CT> n) {
   const bool finite = fabs(n.x + n.y) < CT(INFINITY);
   const bool positive = n.x > CT(0) && n.y > CT(0);
-  if (!finite || (a.self_on && a.psi_exp && !positive)) atomicOr(a.err, 1u);
+  if (!finite || (a.self_on && a.psi_exp && !positive))
+    if (!LOOK || !(*static_cast<volatile unsigned *>(a.err) & 1u)) atomicOr(a.err, 1u);
 }
 
 // Store the post-collision pairs (deviations from w_i nbar).  With a local

@@ -215,7 +215,7 @@ __device__ __forceinline__ void split_collide(const SplitArgs<CT> &m, ST *dst, f
   half_momentum<ST, CT>(j, F, a.inv_scale, h);
   common_velocity<CT>(h, n, u);
   collide_pair<kD3Q19, ST, CT, true>(a, nullptr, n, dn, u, F, out);
-  check_density<CT>(a, n);
+  check_density<CT, true>(a, n);
 #pragma unroll
   for (int i = 0; i < L::Q; ++i)
     Codec2<ST, CT>::store(at(dst + (int64_t)i * a.N * 2, unsigned(s) * unsigned(2 * sizeof(ST))), out[i], a.scale);
