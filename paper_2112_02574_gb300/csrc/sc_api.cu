@@ -123,21 +123,42 @@ bool split_eligible(const sc_params *p) {
   const int64_t site = (p->storage == SC_STORE_F64 ? 16 : 8) * (p->G_self[0] != 0.0 || p->G_self[1] != 0.0 ? 2 : 1);
   return (int64_t)p->nx * p->ny * p->nz <= (int64_t(1) << 32) / site;
 }
-// ... and does: the step kernel is left to the library (no variant, tile or pipeline asked for), and the lattice
-// cannot take the staged kernel, or is FP64 or 16-bit, or is small enough in FP32.  Staged -> two passes, us a step,
-// without a self coupling: FP32 64^3 21.3 -> 11.9, 128^3 120.3 -> 107.8, 160^3 227.9 -> 220.5, 192^3 381.6 -> 380.4,
-// 320^3 1691 -> 1717; FP16 128^3 91.5 -> 80.4, 192^3 286.5 -> 275.9, 256^3 652 -> 636, 320^3 1243 -> 1240; BF16 256^3
-// 648 -> 637, 320^3 1237 -> 1242.  With one, whose psi the staged kernel evaluates again in every halo: FP32 320^3
-// 1837 -> 1782, 512^3 7207 -> 7313; FP16 320^3 1499 -> 1334, 512^3 5717 -> 5511; BF16 512^3 5689 -> 5547.
+// The step kernel is left to the library: no variant, tile or pipeline asked for.
 bool split_asked(const sc_params *p) {
   return split_eligible(p) && !p->variant && !p->tile_y && !p->tile_z && !p->stages && !p->blocks_per_sm;
 }
+// ... and two passes are taken: always where the staged kernel cannot run, in FP64 (64^3 320 -> 212 us a step) and for
+// 16-bit lattices of a few planes, whose periodic z halo the staged kernel sums again for each; else up to the sizes
+// where the staged kernel catches up.  Staged -> two passes, us a step:
+//  * FP32: 64^3 21.3 -> 11.9, 128^3 120.3 -> 107.8, 160^3 227.9 -> 220.7, 168^3 281.4 -> 281.0, 320^3 1691 -> 1717;
+//    with a self coupling, whose psi the staged kernel evaluates again in every halo, 320^3 1841 -> 1784, 328^3
+//    1999 -> 1998, 512^3 7207 -> 7313;
+//  * 16-bit without one (FP16; BF16 within 0.6 %): 128^3 91.5 -> 80.4, 256^3 652 -> 637, 288^3 930 -> 909, 320^3 1245 ->
+//    1246, 384^3 2119 -> 2134, 512^3 4794 -> 5079.  A lattice that fills the tiles of 32 x 8 badly gains longer: 336^3
+//    (95 % of the lanes) 1455 -> 1440, 36 x 898 x 897 (56 %) 1834 -> 1098; one of a single x tile less: 32 x 500 x 500
+//    296 -> 305, 32 x 952 x 952 1016 -> 1079;
+//  * 16-bit with one: 256^3 778 -> 688, 512^3 5717 -> 5511, 640^3 11 121 -> 11 033.
+// The collision reads the densities of three planes; where what two planes stream through L2 exceeds it they come from
+// DRAM again: FP16 with psi 1024 x 1024 x 120 5357 -> 5836, 768 x 768 x 224 5690 -> 5776, without 1024 x 1024 x 16 660 ->
+// 685 (1024 x 1024 x 8, small enough to stay: 364 -> 345); FP32 with psi 768 x 768 x 48 1595 -> 1639.
 bool split_default(const sc_params *p) {
   if (!split_asked(p)) return false;
   if (!use_staged(p) || p->storage == SC_STORE_F64) return true;
-  if (is_16bit(p->storage)) return true;
-  const int64_t sites = (int64_t)p->nx * p->ny * p->nz;
-  return sites <= (has_self(p) ? int64_t(1) << 25 : int64_t(9) << 19);
+  constexpr int64_t M = int64_t(1) << 20;
+  const bool psi = has_self(p), half = is_16bit(p->storage);
+  const int64_t plane = (int64_t)p->nx * p->ny, sites = plane * p->nz;
+  const bool thin = p->nz < (psi ? 16 : 12);
+  if (half && thin) return true;
+  int64_t most = psi ? 32 * M : 9 * M / 2;
+  if (half) {
+    const int64_t lanes = (int64_t)((p->nx + 31) / 32 * 32) * ((p->ny + 7) / 8 * 8);
+    if (psi || plane * 100 < lanes * 93) most = INT64_MAX;
+    else if (plane * 100 < lanes * 97) most = 96 * M;
+    else most = (p->nx == 32 ? 4 : 27) * M;
+  }
+  if (sites > most) return false;
+  const int64_t wide = half ? (psi ? 560000 : 420000) : 300000, kept = (half && psi ? 27 : 12) * M;
+  return thin || plane <= wide || sites <= kept;
 }
 
 sc_status validate(const sc_params *p) {

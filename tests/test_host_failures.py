@@ -215,3 +215,28 @@ def test_large_d2q9_lattices_take_plain_launches(B, L, storage, tau, side, depen
     L.fake_reset()
     assert L.sc_step(c.ctx, 1) == B.SC_OK
     assert [n.endswith("(dependent)") for n in fake_gpu.calls(L)] == [dependent]
+
+
+@pytest.mark.parametrize("storage,psi,shape,passes", [
+    # FP32: 4.7 M sites, 33 M with psi
+    ("F32", False, (160, 160, 160), 2), ("F32", False, (168, 168, 168), 1), ("F32", True, (320, 320, 320), 2),
+    ("F32", True, (324, 324, 324), 1),
+    # 16-bit without psi: full tiles up to 28 M sites, one x tile up to 4 M, partial tiles further
+    ("F16", False, (288, 288, 288), 2), ("BF16", False, (320, 320, 320), 1), ("F16", False, (512, 512, 512), 1),
+    ("F16", False, (32, 360, 360), 2), ("F16", False, (32, 400, 400), 1), ("BF16", False, (336, 336, 336), 2),
+    ("F16", False, (496, 496, 496), 1), ("F16", False, (36, 1200, 1200), 2),
+    # with psi
+    ("F16", True, (512, 512, 512), 2), ("BF16", True, (640, 640, 640), 2),
+    # planes too large for two of them to stay in L2, unless the lattice is small or a few planes thick
+    ("F16", True, (1024, 1024, 120), 1), ("F16", True, (1024, 1024, 16), 2), ("F16", False, (1024, 1024, 16), 1),
+    ("F16", False, (1024, 1024, 8), 2), ("F32", True, (768, 768, 48), 1), ("F32", True, (512, 512, 64), 2),
+    # what the staged kernel cannot take
+    ("F32", False, (321, 320, 320), 2), ("F16", False, (518, 512, 512), 2),
+])
+def test_lone_lattices_take_two_passes_where_they_gain(B, L, storage, psi, shape, passes):
+    c = fake_gpu.Context(L, B.make_params(shape, G=2.5, G_self=(-0.4 if psi else 0.0, 0.0),
+                                          storage=getattr(B, f"SC_STORE_{storage}")))
+    assert c.status == B.SC_OK
+    v = (ctypes.c_int32 * 8)()
+    assert L.sc_step_config(c.ctx, v, 8) == B.SC_OK
+    assert v[0] == passes + 1 if passes == 2 else v[0] == 2
