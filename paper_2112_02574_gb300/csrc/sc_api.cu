@@ -342,6 +342,7 @@ struct sc_batch {
   int split, stencil, storage;
   int *group_at, ngroups;
   int *group_one;  // the member of a group of one large lattice (launched as a lone lattice is), else -1
+  sc_ctx **lone;   // such a member with the step kernel of a lone lattice of its parameters (nullptr: a small one)
   void *sargs_dev;
   int2 *sitems_dev;
   // the persistent form of the staged batch (one cooperative launch runs kGraphSteps steps of every
@@ -568,22 +569,8 @@ SplitArgs<CT> split_args(sc_ctx *c) {
   return m;
 }
 
-// One two-pass step from buffer `swap` on stream st.
-cudaError_t launch_split_step(sc_ctx *c, int swap, cudaStream_t st) {
-  const int sten = c->p.stencil == SC_FORCE_E6 ? kE6 : kE4, cur = c->cur;
-  c->cur = swap;
-  cudaError_t e;
-  switch (c->p.storage) {
-    case SC_STORE_F32: e = launch_split_f32(sten, split_args<float>(c), st); break;
-    case SC_STORE_F16: e = launch_split_f16(sten, split_args<float>(c), st); break;
-    case SC_STORE_BF16: e = launch_split_bf16(sten, split_args<float>(c), st); break;
-    default: e = launch_split_f64(sten, split_args<double>(c), st); break;
-  }
-  c->cur = cur;
-  return e;
-}
-
-sc_status launch_one_step(sc_ctx *c) {
+// One time step of a lattice from buffer `swap` on stream st, by its step kernel.
+cudaError_t launch_step(sc_ctx *c, int swap, cudaStream_t st) {
   StepLaunch l;
   l.lattice = c->p.lattice == SC_D3Q19 ? kD3Q19 : kD2Q9;
   l.stencil = c->p.stencil == SC_FORCE_E6 ? kE6 : kE4;
@@ -592,13 +579,19 @@ sc_status launch_one_step(sc_ctx *c) {
   l.stages = c->stages;
   l.blocks_per_sm = c->blocks_per_sm;
   l.grid = dim3((c->p.nx + 31) / 32, (c->p.ny + c->tile_y - 1) / c->tile_y, (c->p.nz + c->tile_z - 1) / c->tile_z);
-  l.stream = c->stream;
+  l.stream = st;
+  const int cur = c->cur;
+  c->cur = swap;
   cudaError_t e;
   if (c->split) {
-    c->fields_at = -1;  // the moments take the fields' space, also where the collision then fails to launch
-    e = launch_split_step(c, c->cur, c->stream);
+    switch (c->p.storage) {
+      case SC_STORE_F32: e = launch_split_f32(l.stencil, split_args<float>(c), st); break;
+      case SC_STORE_F16: e = launch_split_f16(l.stencil, split_args<float>(c), st); break;
+      case SC_STORE_BF16: e = launch_split_bf16(l.stencil, split_args<float>(c), st); break;
+      default: e = launch_split_f64(l.stencil, split_args<double>(c), st); break;
+    }
   } else if (c->lanes) {
-    e = launch_step_lanes(step_args<double>(c), c->stream);
+    e = launch_step_lanes(step_args<double>(c), st);
   } else {
     switch (c->p.storage) {
       case SC_STORE_F32: e = launch_step_f32(l, step_args<float>(c)); break;
@@ -607,6 +600,13 @@ sc_status launch_one_step(sc_ctx *c) {
       default: e = launch_step_f64(l, step_args<double>(c)); break;
     }
   }
+  c->cur = cur;
+  return e;
+}
+
+sc_status launch_one_step(sc_ctx *c) {
+  if (c->split) c->fields_at = -1;  // the moments take the fields' space, also where the collision then fails to launch
+  const cudaError_t e = launch_step(c, c->cur, c->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();  // reported here, not by the next call
     return fail(SC_ECUDA, "step kernel launch: %s", cudaGetErrorString(e));
@@ -615,6 +615,20 @@ sc_status launch_one_step(sc_ctx *c) {
   c->launches++;
   c->steps++;
   return SC_OK;
+}
+
+// The step kernel of a context and its launch shape; two_pass: the workspace has room for the moments.
+sc_status choose_kernel(sc_ctx *c, bool two_pass) {
+  const sc_params *params = &c->p;
+  c->tile_y = default_tile_y(params);
+  c->tile_z = default_tile_z(params);
+  c->staged = use_staged(params) ? 1 : 0;
+  c->stages = effective_stages(params, c->tile_y);
+  c->blocks_per_sm = effective_blocks_per_sm(params, c->tile_y);
+  c->split = two_pass && split_default(params) ? 1 : 0;
+  c->lanes = use_lanes(params) ? 1 : 0;
+  if (c->lanes) c->tile_y = 1;
+  return !c->split && params->tile_z == 0 && params->lattice == SC_D3Q19 ? plan_z_split(c) : SC_OK;
 }
 
 // Deterministic sums / maxima of the two initial fields.
@@ -698,21 +712,11 @@ sc_status create_context(const sc_params *params, const double *nA0, const doubl
   c->ws = static_cast<char *>(workspace);
   c->L = L;
   c->cur = 0;
-  c->tile_y = default_tile_y(params);
-  c->tile_z = default_tile_z(params);
-  c->staged = use_staged(params) ? 1 : 0;
-  c->stages = effective_stages(params, c->tile_y);
-  c->blocks_per_sm = effective_blocks_per_sm(params, c->tile_y);
   c->fields_at = -1;
-  c->split = two_pass && split_default(params) ? 1 : 0;
-  c->lanes = use_lanes(params) ? 1 : 0;
-  if (c->lanes) c->tile_y = 1;
-  if (!c->split && params->tile_z == 0 && params->lattice == SC_D3Q19) {
-    st = plan_z_split(c);
-    if (st != SC_OK) {
-      delete c;
-      return st;
-    }
+  st = choose_kernel(c, two_pass);
+  if (st != SC_OK) {
+    delete c;
+    return st;
   }
   double mean[2], maxdev[2];
   cudaError_t e = cudaMemsetAsync(c->ws + L.off_status, 0, kStatusBytes, c->stream);
@@ -1204,6 +1208,9 @@ bool batch_split(int32_t n, const sc_params *params) {
 // The members of a two-pass batch that have fewer sites than this step in groups of at least this many, the others
 // alone, each group through all the steps of a run before the next: the lattices are independent, a group this
 // size fills the GPU, and its moments (and part of its populations) stay in L2 from one pass to the next.
+// A 16-bit member alone takes the step kernel of a lone lattice of its parameters (split_default): one of 512^3 without
+// psi 5094 -> 4799 us a step.  The others take two passes: FP32 without psi 2 x 320^3 3383 -> 3435 against the staged
+// kernel's single launches (4157 its persistent ones), 512^3 7736 -> 6961.
 // Us a step, one launch per pass for all -> groups: 14 paper droplets (1.5 M sites) FP32 95.0 -> 87.3, FP16 78.3 -> 73.4;
 // 8 droplets (1.9 M) FP32 108.5 -> 99.4; 16 droplets (22.1 M, mostly large members) FP32 1234 -> 1225, FP16 1006 -> 994.
 constexpr int64_t kGroupSites = 768 << 10;
@@ -1383,7 +1390,7 @@ bool batch_build_persistent(sc_batch *b) {
 
 // One time step of group g of a two-pass batch on stream st.
 cudaError_t batch_split_step(const sc_batch *b, int g, int swap, cudaStream_t st) {
-  if (b->group_one[g] >= 0) return launch_split_step(b->ctx[b->group_one[g]], swap, st);
+  if (b->group_one[g] >= 0) return launch_step(b->lone[b->group_one[g]], swap, st);
   const int2 *items = b->sitems_dev + b->group_at[g];
   const int n = b->group_at[g + 1] - b->group_at[g];
   const SplitArgs<float> *af = static_cast<SplitArgs<float> *>(b->sargs_dev);
@@ -1557,9 +1564,22 @@ sc_status sc_batch_create(int32_t n, const sc_params *params, const double *cons
   b->retired = new (std::nothrow) char[n];
   b->group_at = new (std::nothrow) int[n + 1];
   b->group_one = new (std::nothrow) int[n];
-  if (!b->retired || !b->group_at || !b->group_one) {
+  b->lone = new (std::nothrow) sc_ctx *[n]();
+  if (!b->retired || !b->group_at || !b->group_one || !b->lone) {
     sc_batch_destroy(b);
     return fail(SC_ENOMEM, "host allocation failed");
+  }
+  for (int k = 0; k < n && b->split; ++k) {
+    if (b->ctx[k]->N < kGroupSites) continue;
+    sc_ctx *c = new (std::nothrow) sc_ctx(*b->ctx[k]);
+    b->lone[k] = c;
+    if (c) c->p = params[k];
+    st = c ? choose_kernel(c, true) : fail(SC_ENOMEM, "host allocation failed");
+    if (c && !is_16bit(storage)) c->split = 1;
+    if (st != SC_OK) {
+      sc_batch_destroy(b);
+      return st;
+    }
   }
   memset(b->retired, 0, n);
   b->active = n;
@@ -1727,6 +1747,9 @@ void sc_batch_destroy(sc_batch *b) {
   delete[] b->retired;
   delete[] b->group_at;
   delete[] b->group_one;
+  if (b->lone)
+    for (int k = 0; k < b->n; ++k) delete b->lone[k];
+  delete[] b->lone;
   delete b;
 }
 

@@ -240,3 +240,22 @@ def test_lone_lattices_take_two_passes_where_they_gain(B, L, storage, psi, shape
     v = (ctypes.c_int32 * 8)()
     assert L.sc_step_config(c.ctx, v, 8) == B.SC_OK
     assert v[0] == passes + 1 if passes == 2 else v[0] == 2
+
+
+def test_large_batch_members_take_their_lone_kernel(B, L):
+    """A 16-bit member that steps alone in a two-pass batch does so as a lone lattice of its parameters would: one staged
+    launch a step where that one would not take two passes.  In FP32 it takes two passes at any size."""
+    for storage, staged in (("F16", True), ("F32", False)):
+        kw = dict(G=2.5, storage=getattr(B, f"SC_STORE_{storage}"))
+        b = fake_gpu.Batch(L, [B.make_params(s, **kw) for s in ((16, 16, 16), (32, 400, 400), (96, 96, 96))])
+        assert b.status == B.SC_OK and L.sc_batch_variant(b.handle) == 4
+        L.fake_reset()
+        assert L.sc_batch_step(b.handle, 1) == B.SC_OK
+        two = ["split_moments", "split_collide"]
+        kinds = ("split_moments_batched", "split_collide_batched", *two, "step_staged")
+        assert [next(k for k in kinds if k in n) for n in fake_gpu.calls(L)] == [
+            *kinds[:2], *(["step_staged"] if staged else two), *two]
+        assert L.sc_batch_retire(b.handle, 1) == B.SC_OK
+        L.fake_reset()
+        assert L.sc_batch_step(b.handle, 1) == B.SC_OK
+        assert not any("staged" in n for n in fake_gpu.calls(L)) and len(fake_gpu.calls(L)) == 4
