@@ -123,11 +123,14 @@ sc_status sc_create(const sc_params *params, const double *nA0, const double *nB
 /* Advance nsteps >= 0 time steps of Eq. lbm (BGK of Eq. omega_i, Guo forcing,
  * equilibrium of Eq. feq, common velocity of Eq. u, force of Eq. sc_force,
  * streaming).  One fused kernel launch per step, or two (a moments pass and a
- * collision pass, the library's choice for small, odd, E6 and FP64 lattices with
- * tau = 1); asynchronous.  Runs of 32 steps are replayed from a CUDA graph that
- * the context captures once, on a private stream, the first time such a run comes
- * up (the replay goes to the context's stream; if the capture is not possible the
- * steps are plain launches). */
+ * collision pass: the library's choice with tau = 1 for E6, FP64 and odd lattices,
+ * most 16-bit ones and the smaller FP32 ones; sc_step_config tells); asynchronous.
+ * Runs of 32 steps are replayed from a CUDA graph that the context captures once,
+ * on a private stream, the first time such a run comes up (the replay goes to the
+ * context's stream; if the capture is not possible the steps are plain launches).
+ * Fewer steps than that may be recorded into a caller's graph; what is read after
+ * a replay is the state it left (record an even number of steps: a step swaps the
+ * two buffers, and the context counts a recorded step once). */
 sc_status sc_step(sc_ctx *ctx, int64_t nsteps);
 
 /* Densities n_A, n_B (device FP64 [N] each) and, if u != NULL, the common
@@ -312,15 +315,15 @@ sc_status sc_run_host_sigma(const sc_params *params, const double *nA0, const do
 /* ---- batches: several lattices stepped together ----
  * The batched radius sweep: lattices of different sizes and parameters (same
  * lattice type, stencil, storage and tile_y) stepped together over a work list
- * of (lattice, tile) items, from a CUDA graph (built explicitly, no stream
- * capture).  The kernel is the staged one when every member can take it
+ * of (lattice, tile) items, from a CUDA graph (built node by node; for two passes
+ * captured on a private stream, and plain launches where that fails).  The kernel is the staged one when every member can take it
  * (variant 0 or 2, D3Q19, E4, nx >= 32 a multiple of the chunk sites; members
  * then share stages and blocks_per_sm), else the generic one; a member with
  * variant 2 in a batch that cannot be staged is an error (SC_EINVAL).  Where every
  * member leaves variant, tiles and pipeline to the library, is D3Q19 with tau = 1
  * and has sides >= 4, the batch steps in two passes (a moments and a collision
- * launch per step, replayed from a CUDA graph) unless a persistent launch is asked
- * for (sc_batch_set_persistent).
+ * launch per step for each group of small members and for each large one) unless a
+ * persistent launch is asked for (sc_batch_set_persistent).
  * By default (where the device has cooperative launch; see
  * sc_batch_set_persistent) a staged batch that does not step in two passes runs 32
  * time steps of every member in ONE persistent cooperative launch: in each step its blocks draw the work

@@ -1,7 +1,8 @@
 // Kernels around the time step: initial state, population access, FP64
 // density / pseudopotential fields, the common velocity, the lattice pressure
 // tensor with its profiles, the sigma[R] minimum and conserved totals.
-// All analysis arithmetic is FP64 (arXiv:2112.02574, sections 2 and 3).
+// Analysis results are FP64 (arXiv:2112.02574, sections 2 and 3): sums of stored values are three-term FP32 expansions
+// of FP64 accuracy (PairSum3), the sigma[R] grid is screened in FP32, everything else is FP64 arithmetic.
 #pragma once
 
 #include "sc_common.cuh"
@@ -259,7 +260,7 @@ __device__ __forceinline__ void gradient64(const double *f, int s, const int *X,
 
 // Common velocity of Eq. u (force of Eq. sc_force included) at site s, FP64.  With both self couplings the four
 // fields' differences across a stencil pair, each with its own factor, add up before they meet the pair's vector:
-// 87 FP64 instructions instead of 108 for four gradients (convergence check of 14 droplets 1430 -> 1323 us).  With
+// 87 FP64 instructions instead of 108 for four gradients (convergence check of 14 droplets 1430 -> 1333 us).  With
 // three fields the longer chain costs more than the 12 instructions it saves (fields and diagnostics at 128^3
 // 2690 -> 2745 us), so each has its own gradient there.
 template <int LAT, int STEN, class ST>
@@ -450,8 +451,9 @@ __global__ void bulk_pressure_kernel(ForceParams fp, const double *fields, int64
 // sigma[R] minimum (section 3) on one block of 256 threads (one warp for at most 32 rows and samples); see sc_sigma_minimum in sc.h.
 //  * The trapezoid of r^(dim-1) P_T: rows come 256 at a time into shared memory, every thread forms the term of its
 //    row with the last non-empty row before it, and the terms are added in a fixed tree.
-//  * The grid search needs sigma[R] in FP64 only where it can be the minimum: FP32 values of all samples, good to
-//    1e-5 of the sizes of their two terms, leave those whose lower bound is below every upper bound.
+//  * The grid search needs sigma[R] in FP64 only where it can be the minimum: FP32 values of all samples leave those
+//    whose lower bound is below every upper bound.  Their margin is 1e-5 of the sizes of the two terms; R = lo + k step
+//    (k < 2^24 exact, both summands positive) and the two terms take at most ten roundings of 2^-24 each, 6e-7.
 // One warp did both one after another before: 212 us at 128 rows and 6400 samples, now 18 us.  The trees and the
 // search for a chunk's last row span the rows and samples there are: 2 rows and 5 samples 18.9 -> 11.3 us (9.8 in the
 // one warp).

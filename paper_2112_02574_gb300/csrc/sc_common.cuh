@@ -260,7 +260,7 @@ __host__ __device__ constexpr bool local_ref() {
   return sizeof(ST) == 2;
 }
 
-// Exact quotient of 0 <= n < 2^31 by a fixed divisor: mul = ceil(2^(32 + shift) / div), shift =
+// Exact quotient of 0 <= n < 2^31 by a fixed divisor (Granlund and Montgomery's multiplication by the reciprocal): mul = ceil(2^(32 + shift) / div), shift =
 // ceil(log2 div) - 1, so that the rounding of mul adds less than 1 / div to n / div.
 struct FastDiv {
   unsigned mul, shift, div;

@@ -1,4 +1,5 @@
-// The time step in two passes (D3Q19, E4 or E6, tau_A = tau_B = 1, every side >= 4, any storage).
+// The time step in two passes (D3Q19, E4 or E6, tau_A = tau_B = 1, every side >= 4, any storage); split_default in
+// sc_api.cu says which lattices take it.
 //
 //  * The moments pass pulls the populations of a site once and keeps what collisions need of them:
 //    the density deviation pair, the three momentum-sum pairs (carry_size) and, with a self coupling,
@@ -15,7 +16,8 @@
 // Measured, one step, one-pass -> two passes (FP32 unless noted): E6 64 x 64 x 256 80.3 -> 58.0 us,
 // E6 160^3 302 -> 259 us (FP16 363 -> 209 us), 65^3 29.5 -> 14.9 us (paper couplings), 201^3 567 -> 499 us,
 // 64^3 21.4 -> 12.0 us, FP64 64^3 320 -> 212 us (one psi).  Bound: HBM at large sizes (256^3: 368 bytes a site at
-// 6.9 TB/s), FP64 arithmetic in FP64, latency below about 40^3.
+// 6.9 TB/s; 512^3 FP16 with psi: 248 bytes a site, 80 of them moments, at 6.0 TB/s), FP64 arithmetic in FP64, latency
+// below about 40^3.
 #pragma once
 
 #include "sc_step_kernel.cuh"
@@ -35,7 +37,7 @@ struct SplitArgs {
 
 // L2 eviction priorities.  The moments are written by one pass and read by the next; the populations of a large
 // lattice stream through L2 in between and would push them out, though the next step cannot find them there
-// either.  Where the moments fit in L2 (keep_moments) they are written with evict-last, the populations are read
+// either.  Up to a measured size (keep_moments, kKeptMoments in sc_api.cu) they are written with evict-last, the populations are read
 // with evict-first, and so are the momentum sums, for the last time, so that no evict-last line of theirs is left
 // behind.  Us a step, all normal -> so: E6 64 x 64 x 256 67.8 -> 59.4, 96^3 FP32 51.5 -> 42.1,
 // 128^3 FP32 117.9 -> 108.2, FP16 94.1 -> 88.6, 160^3 FP32 (131 MB of moments) 227.5 -> 221.8; no effect at 64^3

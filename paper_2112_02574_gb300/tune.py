@@ -74,7 +74,7 @@ def tune_batch(params_list, fields, candidates, steps: int = 32, device="cuda"):
     """(tile_y, tile_z, stages, blocks_per_sm, persistent) for a batch (shared by its members), timed on
     the whole batch: each candidate block shape with whole 32-step runs as one persistent launch (where
     the batch has that form) and as one launch per step (steps a multiple of 32 times the graph
-    replays).  Returns (best, ms_per_step, table)."""
+    replays); a candidate that leaves the kernel to the library times its two passes.  Returns (best, ms_per_step, table)."""
     table = []
     for cfg in candidates:
         batch = B.Batch([with_config(p, cfg) for p in params_list], fields, device=device)
