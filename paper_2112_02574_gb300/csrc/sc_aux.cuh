@@ -401,11 +401,17 @@ __device__ __forceinline__ void block_rows_sum(const double *partial, int nblock
 #pragma unroll
   for (int c = 0; c < NC; ++c) red[c][threadIdx.x] = acc[c];
   __syncthreads();
-  for (int w = tree_top(nblocks); w > 0; w >>= 1) {
+  auto halve = [&](int w) {
     if (threadIdx.x < w)
 #pragma unroll
       for (int c = 0; c < NC; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + w];
     __syncthreads();
+  };
+  if (nblocks > 128) {
+#pragma unroll
+    for (int w = 128; w > 0; w >>= 1) halve(w);
+  } else {
+    for (int w = tree_top(nblocks); w > 0; w >>= 1) halve(w);
   }
 #pragma unroll
   for (int c = 0; c < NC; ++c) out[c] = red[c][0];

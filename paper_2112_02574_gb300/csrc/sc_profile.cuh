@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(256) profile_partial_kernel(ForceParams fp, Pr
   double *out = partial + (int64_t)blockIdx.x * row;
   const double *all = reinterpret_cast<const double *>(smem_raw);
   if constexpr (RADIAL) {
-    if (nwarps == 1) {  // many bins: a plain copy, whose loads the loop overlaps
+    if (nwarps == 1 && pa.nbins >= 1024) {  // a plain copy, whose loads the loop overlaps
 #pragma unroll 8
       for (int k = lane; k < row; k += 32) out[k] = all[k];
       return;
